@@ -96,6 +96,8 @@ void free_mg(lm_grid* g) {
     }
     g->mg.clear();
     g->mg_built = false;
+    cudaFree(g->cc_plan);
+    g->cc_plan = nullptr;
 }
 
 bool mg_supported(const lm_grid* g) {
@@ -112,8 +114,25 @@ int build_mg(lm_grid* g, cudaStream_t s, bool defer_inverse = false) {
         g->inv_pending = defer_inverse;
         if (!defer_inverse) launch_coarse_inverse(Lc.L, s, Lc.ainv);
     };
+    // likewise the plan of the one-launch coarse cycle (a batch forms its own)
+    auto plan = [&]() -> int {
+        g->plan_pending = defer_inverse;
+        if (defer_inverse || g->cc_level < 0) return LM_OK;
+        size_t smem = 0, size = 0;
+        auto chain = [&]() {
+            return lm::coarse_chain(g, g->cc_level, g->cc_blocks, true, g->cc_plan, nullptr, nullptr, 1, 1, &smem, &size);
+        };
+        if (!g->cc_plan) {
+            chain();
+            if (int rc = dalloc(&g->cc_plan, size)) return rc;
+        }
+        launch_cc_plan(chain(), s);
+        return LM_OK;
+    };
+    int rc;
     if (g->mg_built) {
         if (g->inv_pending && !defer_inverse) inverse(g->mg.back());
+        if (g->plan_pending && !defer_inverse && (rc = plan())) return rc;
         CK(cudaGetLastError());
         return LM_OK;
     }
@@ -127,6 +146,7 @@ int build_mg(lm_grid* g, cudaStream_t s, bool defer_inverse = false) {
         }
         MgLevel& Lc = g->mg.back();
         if (Lc.ainv) inverse(Lc);
+        if ((rc = plan())) return rc;
         CK(cudaGetLastError());
         g->mg_built = true;
         return LM_OK;
@@ -157,7 +177,6 @@ int build_mg(lm_grid* g, cudaStream_t s, bool defer_inverse = false) {
             F.halved[a] = hv[a];
         }
         const int Nc = nc[0] * nc[1] * nc[2];
-        int rc;
         if ((rc = dalloc(&C.ct, Nc)) || (rc = dalloc(&C.rho, Nc)) || (rc = dalloc(&C.xa, Nc)) ||
             (rc = dalloc(&C.xb, Nc)) || (rc = dalloc(&C.xo, Nc)) || (rc = dalloc(&C.f, Nc)))
             return rc;
@@ -167,25 +186,23 @@ int build_mg(lm_grid* g, cudaStream_t s, bool defer_inverse = false) {
     }
     MgLevel& Lc = g->mg.back();
     if (Lc.L.g.N <= COARSE_EXACT) {
-        int rc = dalloc(&Lc.ainv, (size_t)Lc.L.g.N * Lc.L.g.N);
-        if (rc) return rc;
+        if ((rc = dalloc(&Lc.ainv, (size_t)Lc.L.g.N * Lc.L.g.N))) return rc;
         inverse(Lc);
     }
-    // the one-block coarse V-cycle takes over from the first level small
-    // enough, when the chain ends in a directly solved level
-    g->cc_level = -1;
+    // A hierarchy solved exactly at the bottom smooths its last levels (at
+    // most five, from 4096 cells, 28 bytes a cell in 200 KB) with the correctly
+    // rounded inverse diagonal, every other level with an approximate division.
+    g->inverse_level = -1;
     if (g->mg.back().ainv)
-        for (size_t l = 0; l < g->mg.size(); ++l)
-            if (g->mg[l].L.g.N <= CC_MAX_CELLS && g->mg.size() - l <= (size_t)CC_MAXL && g->mg.size() - l >= 2) {
-                int N[CC_MAXL];
-                const int nl = (int)(g->mg.size() - l);
-                for (int i = 0; i < nl; ++i) N[i] = g->mg[l + i].L.g.N;
-                if (cc_smem_bytes(N, nl) <= CC_SMEM_MAX) {
-                    coarse_cycle_allow_smem();
-                    g->cc_level = (int)l;
-                }
-                break;
-            }
+        for (size_t l = 0; l + 2 <= g->mg.size(); ++l) {
+            if (g->mg[l].L.g.N > 4096 || g->mg.size() - l > 5) continue;
+            size_t bytes = sizeof(float) * (size_t)g->mg.back().L.g.N * g->mg.back().L.g.N;
+            for (size_t k = l; k < g->mg.size(); ++k) bytes += 7 * sizeof(float) * (size_t)g->mg[k].L.g.N;
+            if (bytes <= 200 * 1024) g->inverse_level = (int)l;
+            break;
+        }
+    g->cc_level = lm::chain_level(g, g->cc_blocks);
+    if ((rc = plan())) return rc;
     CK(cudaGetLastError());
     g->mg_built = true;
     return LM_OK;
@@ -220,21 +237,9 @@ float* sweep_chain(MgLevel& M, cudaStream_t s, int count, const int* first, cons
 void vcycle(lm_grid* g, int l, float* xout, const float* f, int nu1, int nu2, cudaStream_t s) {
     MgLevel& M = g->mg[l];
     if (l == g->cc_level) {          // the rest of the cycle in one block
-        CoarseCycle cc{};
-        cc.nl = (int)g->mg.size() - l;
-        for (int i = 0; i < cc.nl; ++i) {
-            const MgLevel& Li = g->mg[l + i];
-            cc.L[i] = Li.L;
-            cc.hx[i] = Li.halved[0];
-            cc.hy[i] = Li.halved[1];
-            cc.hz[i] = Li.halved[2];
-            cc.x[i] = i == 0 ? xout : Li.xo;
-            cc.f[i] = i == 0 ? const_cast<float*>(f) : Li.f;
-        }
-        cc.ainv = g->mg.back().ainv;
-        cc.nu1 = nu1;
-        cc.nu2 = nu2;
-        launch_coarse_cycle(cc, s);
+        size_t smem = 0;
+        const CoarseCycle cc = lm::coarse_chain(g, l, g->cc_blocks, true, g->cc_plan, xout, f, nu1, nu2, &smem);
+        launch_coarse_cycle(cc, smem, s);
         return;
     }
     const bool last = (size_t)l + 1 == g->mg.size();
@@ -842,6 +847,67 @@ int lm::grid_finish_assembly(lm_grid* g, const AsmFlags& fl, cudaStream_t s) {
     return LM_OK;
 }
 
+// swept by zrow2d_tile when on its own
+static bool axis_arith(const Geo& g) { return g.ny == 1 && g.nx % 128 == 0 && g.nz >= 2; }
+// swept by k_rbgs_zm or k_rbgs_row when on its own
+static bool march_arith(const Geo& g) { return g.ny > 1 && g.nx % 32 == 0 && g.ny % 8 == 0 && g.nz >= 2; }
+
+int lm::chain_level(const lm_grid* g, int nr_max) {
+    const int nl = (int)g->mg.size();
+    for (int l = std::max(0, nl - CC_MAXL); l < nl; ++l) {
+        if (l + 1 == nl && g->mg[l].ainv) break;               // the dense inverse alone: k_coarse_solve
+        size_t smem = 0;
+        const CoarseCycle cc = coarse_chain(g, l, nr_max, true, nullptr, nullptr, nullptr, 1, 1, &smem);
+        bool fits = smem <= CC_SMEM_MAX;
+        for (int k = 0; k < cc.nl; ++k) {
+            const CCLevel& v = cc.lev[k];
+            const Geo& q = v.L.g;
+            fits = fits && v.hp * q.ny * cc_own(v) <= CC_THREADS * (v.nr > 1 ? CC_PER_SHARED : CC_PER);
+            // a 3D level of whole 32 x 8 tiles marches with kernels of its own,
+            // as does a 2D level of 128-cell segments under a 3D one
+            if (v.arith != CC_INVERSE && march_arith(q)) fits = false;
+            if (cc.lev[0].L.g.ny > 1 && v.arith == CC_AXIS) fits = false;
+            // rbgs_tile leaves the first-colour halo cell beside an x wall, or
+            // of a single-cell row, at its old value where a tile ends in y:
+            // another smoother, which such levels keep
+            if (v.arith == CC_FACE && q.ny > 1 && ((q.bcx == LM_BC_NEUMANN && q.ny > 8) || q.nx == 1)) fits = false;
+        }
+        if (fits) return l;
+    }
+    return -1;
+}
+
+CoarseCycle lm::coarse_chain(const lm_grid* g, int lev, int nr_max, bool inverse, float4* plan, float* x,
+                             const float* f, int nu1, int nu2, size_t* smem, size_t* plan_size) {
+    CoarseCycle cc{};
+    cc.nl = (int)g->mg.size() - lev;
+    size_t size = 0;
+    const int inv = inverse && g->inverse_level >= 0 ? g->inverse_level : (int)g->mg.size();
+    for (int i = 0; i < cc.nl; ++i) {
+        const MgLevel& M = g->mg[lev + i];
+        CCLevel& v = cc.lev[i];
+        v.L = M.L;
+        v.hx = M.halved[0];
+        v.hy = M.halved[1];
+        v.hz = M.halved[2];
+        // one block while the level's pairs fit its registers, else as many
+        // as the cluster has, but no more than units of planes
+        v.nr = cc_pairs(M.L.g) <= CC_MAX_PAIRS ? 1 : std::min(nr_max, M.L.g.nz >> v.hz);
+        v.plan = plan ? plan + size : nullptr;
+        size += (size_t)CC_PLAN * cc_pairs(M.L.g);
+        v.arith = lev + i >= inv ? CC_INVERSE : (axis_arith(M.L.g) ? CC_AXIS : CC_FACE);
+    }
+    cc.x = x;
+    cc.f = f;
+    cc.ainv = g->mg.back().ainv;
+    cc.parts = inv < (int)g->mg.size() ? 16 : 1;
+    cc.nu1 = nu1;
+    cc.nu2 = nu2;
+    *smem = cc_layout(cc);
+    if (plan_size) *plan_size = size;
+    return cc;
+}
+
 int lm::grid_build_mg(lm_grid* g, cudaStream_t s, bool defer_inverse) { return build_mg(g, s, defer_inverse); }
 lm::Lev32 lm::make_level(const int n[3], const int bc[3], const double h[3], const float* ct, const float* rho,
                          double rho_scale) {
@@ -913,7 +979,7 @@ int lm_grid_create(int ndim, const int64_t n[3], const double h[3], const int bc
     // the whole-row and one-block coarse-cycle kernels need more than the
     // default 48 KB of shared memory: allow it before any entry point launches them
     rbgs_row_allow_smem();
-    coarse_cycle_allow_smem();
+    g->cc_blocks = coarse_cycle_allow();
     int nsm = 1;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device);
     const long long want = (N + NT - 1) / NT;

@@ -32,6 +32,7 @@
 #include "lm_internal.h"
 #include "lm_kernels.h"
 #include "lm_tiles.cuh"
+#include "lm_coarse.cuh"
 
 namespace lm {
 
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(256) kb_resid_restrict(const BTask* __restrict
 __global__ void __launch_bounds__(CC_THREADS, 1) kb_coarse_cycle(const CoarseCycle* __restrict__ ccs,
                                                         const BGrid* __restrict__ Gs) {
     if (inner_off(Gs[blockIdx.x])) return;
-    coarse_cycle_block(ccs[blockIdx.x]);
+    coarse_cycle_block<1, false>(ccs[blockIdx.x]);
 }
 
 __global__ void kb_coarse(const BTask* __restrict__ T, const BGrid* __restrict__ Gs, const BLev* __restrict__ Ls) {
@@ -585,6 +586,7 @@ struct Plan {
     int n_inv_tasks = 0;
     CoarseCycle* dcc = nullptr;          // per-grid one-block coarse cycles (null: per-level launches)
     size_t cc_smem = 0;                  // their dynamic shared memory (the largest chain's)
+    float4* dplan = nullptr;             // their plans, formed at every solve
     int max_depth = 0;
     long long n_first = 0, n_step = 0;   // kernels per graph launch (n_step: outside the inner loop)
     long long n_iter = 0;                // kernels per inner iteration of the device-side loop
@@ -600,6 +602,7 @@ struct Plan {
         cudaFree(dlev0);
         cudaFree(dtasks);
         cudaFree(dcc);
+        cudaFree(dplan);
         cudaFree(dinv_items);
         cudaFree(dinv_tasks);
         cudaFree(dgather);
@@ -737,35 +740,29 @@ int build_plan(lm_grid* const* grids, int count, const lm_solve_opts* o, cudaStr
     tap.n = (int)tasks.size() - tap.off;
     // one-block coarse cycles when every grid's hierarchy has one: the
     // per-level task lists then stop at each grid's coarse-cycle level
-    bool fused = true;
+    bool fused = true, inverse = true;
     std::vector<int> lstop(count);
     for (int i = 0; i < count; ++i) {
-        fused = fused && grids[i]->cc_level >= 0;
+        fused = fused && chain_level(grids[i], 1) >= 0;
+        inverse = inverse && grids[i]->inverse_level >= 0;
         lstop[i] = nlev[i] - 1;
     }
     if (fused) {
         std::vector<CoarseCycle> hcc(count);
-        for (int i = 0; i < count; ++i) {
-            lm_grid* g = grids[i];
-            const int lc = g->cc_level;
-            lstop[i] = lc;
-            CoarseCycle& cc = hcc[i];
-            cc = CoarseCycle{};
-            cc.nl = (int)g->mg.size() - lc;
-            for (int k = 0; k < cc.nl; ++k) {
-                const MgLevel& Mk = g->mg[lc + k];
-                cc.L[k] = Mk.L;
-                cc.hx[k] = Mk.halved[0];
-                cc.hy[k] = Mk.halved[1];
-                cc.hz[k] = Mk.halved[2];
-                cc.x[k] = (lc + k == 0) ? g->z32 : Mk.xo;
-                cc.f[k] = (lc + k == 0) ? g->r32 : Mk.f;
+        std::vector<size_t> at(count + 1, 0);
+        for (int pass = 0; pass < 2; ++pass) {           // sizes of the plans, then the chains
+            for (int i = 0; i < count; ++i) {
+                lm_grid* g = grids[i];
+                const int lc = lstop[i] = chain_level(g, 1);
+                size_t smem = 0, size = 0;
+                hcc[i] = coarse_chain(g, lc, 1, inverse, pass ? P->dplan + at[i] : nullptr,
+                                      lc == 0 ? g->z32 : g->mg[lc].xo, lc == 0 ? g->r32 : g->mg[lc].f, o->nu1, o->nu2,
+                                      &smem, &size);
+                P->cc_smem = std::max(P->cc_smem, smem);
+                at[i + 1] = at[i] + size;
             }
-            cc.ainv = g->mg.back().ainv;
-            cc.nu1 = o->nu1;
-            cc.nu2 = o->nu2;
+            if (pass == 0) BCK(cudaMalloc(&P->dplan, sizeof(float4) * std::max<size_t>(at[count], 1)));
         }
-        for (const CoarseCycle& cc : hcc) P->cc_smem = std::max(P->cc_smem, cc_smem_bytes(cc));
         BCK(cudaFuncSetAttribute(kb_coarse_cycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM_MAX));
         BCK(cudaMalloc(&P->dcc, sizeof(CoarseCycle) * count));
         BCK(cudaMemcpy(P->dcc, hcc.data(), sizeof(CoarseCycle) * count, cudaMemcpyHostToDevice));
@@ -1033,6 +1030,7 @@ int batch_refresh(lm_grid* const* grids, int count, cudaStream_t s) {
     for (lm_grid* g : todo) {
         g->mg_built = true;
         if (g->mg.back().ainv) g->inv_pending = true;
+        g->plan_pending = true;
     }
     return LM_OK;
 }
@@ -1142,6 +1140,7 @@ int lm_batch_solve(lm_grid* const* grids, int count, const lm_solve_opts* o, lm_
             for (int i = 0; i < count; ++i) grids[i]->inv_pending = false;
         }
     }
+    if (P->dcc) launch_cc_plan_many(P->dcc, count, s);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);

@@ -12,6 +12,7 @@
 #include "lm_common.cuh"
 #include "lm_kernels.h"
 #include "lm_tiles.cuh"
+#include "lm_coarse.cuh"
 
 namespace lm {
 
@@ -1440,16 +1441,18 @@ __global__ void k_coarse_solve(int n, const float* __restrict__ ainv, const floa
     coarse_solve_block(n, ainv, f, x);
 }
 
-// ---- the coarse V-cycle in one block ------------------------------------------
-// The V-cycle below a level of at most CC_MAX_CELLS cells, run by one block of
-// 1024 threads: per level, nu1 red-black sweeps from zero (in place, the two
-// colours separated by a barrier, so the result equals the fused sweeps'),
-// the residual restricted to the next level's rhs, recursion, then the
-// prolonged correction and nu2 black-red sweeps; the coarsest level is
-// solved with its dense inverse.  Replaces ~3 launches per level and sweep
-// that are all latency-bound at these sizes; the chain lives in shared memory
-// (cc_smem_bytes), so only the setup and the final store touch global memory.
-__global__ void __launch_bounds__(CC_THREADS, 1) k_coarse_cycle(CoarseCycle cc) { coarse_cycle_block(cc); }
+// ---- the coarse V-cycle in one launch (lm_coarse.cuh) ---------------------------
+template <int NR, bool Y3>
+__global__ void __launch_bounds__(CC_THREADS, 1) k_coarse_cycle(const __grid_constant__ CoarseCycle cc) {
+    coarse_cycle_block<NR, Y3>(cc);
+}
+__global__ void __launch_bounds__(128) k_cc_plan(const __grid_constant__ CoarseCycle cc) {
+    cc_plan_range(cc, blockIdx.x * 128 + threadIdx.x, gridDim.x * 128);
+}
+// many grids' chains: row y of the launch plans chain y
+__global__ void __launch_bounds__(128) k_cc_plan_many(const CoarseCycle* __restrict__ ccs) {
+    cc_plan_range(ccs[blockIdx.y], blockIdx.x * 128 + threadIdx.x, gridDim.x * 128);
+}
 
 // ---- host launchers -----------------------------------------------------------
 
@@ -1987,12 +1990,62 @@ void launch_rbgs(const Lev32& L, cudaStream_t s, const float* xin, const float* 
                  int hz, const float* f, float* xout, int first, int zero, int prolong) {
     launch_rbgs_kz(L, s, xin, ec, C, hx, hy, hz, f, xout, first, zero, prolong, 0);
 }
-void coarse_cycle_allow_smem() {
-    cudaFuncSetAttribute(k_coarse_cycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM_MAX);
+static cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t s, cudaLaunchAttribute* attr) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = CC_CLUSTER;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(CC_CLUSTER);
+    c.blockDim = dim3(CC_THREADS);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return c;
 }
-void launch_coarse_cycle(const CoarseCycle& cc, cudaStream_t s) {
+int coarse_cycle_allow() {
+    const void* const ks[] = {(const void*)k_coarse_cycle<1, false>, (const void*)k_coarse_cycle<1, true>,
+                              (const void*)k_coarse_cycle<CC_CLUSTER, false>,
+                              (const void*)k_coarse_cycle<CC_CLUSTER, true>};
+    int n = 0;
+    for (int v = 0; v < 4; ++v) {
+        cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM_MAX);
+        if (v < 2) continue;
+        cudaFuncSetAttribute(ks[v], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t c = cluster_config(CC_SMEM_MAX, nullptr, &attr);
+        int m = 0;
+        if (cudaOccupancyMaxActiveClusters(&m, ks[v], &c) != cudaSuccess) {
+            cudaGetLastError();
+            m = 0;
+        }
+        n = v == 2 ? m : std::min(n, m);
+    }
+    return n > 0 ? CC_CLUSTER : 1;
+}
+void launch_cc_plan(const CoarseCycle& cc, cudaStream_t s) {
+    int pairs = 0;
+    for (int l = 0; l < cc.nl; ++l) pairs += cc_pairs(cc.lev[l].L.g);
     count_launches(1);
-    k_coarse_cycle<<<1, CC_THREADS, cc_smem_bytes(cc), s>>>(cc);
+    k_cc_plan<<<std::min(hdiv(pairs, 128), 8 * 152), 128, 0, s>>>(cc);
+}
+void launch_cc_plan_many(const CoarseCycle* ccs, int count, cudaStream_t s) {
+    if (count <= 0) return;
+    count_launches(1);
+    k_cc_plan_many<<<dim3(hdiv(CC_MAX_PAIRS, 128), count), 128, 0, s>>>(ccs);
+}
+void launch_coarse_cycle(const CoarseCycle& cc, size_t smem, cudaStream_t s) {
+    count_launches(1);
+    const bool y3 = cc.lev[0].L.g.ny > 1;
+    if (cc.lev[0].nr == 1) {
+        if (y3) k_coarse_cycle<1, true><<<1, CC_THREADS, smem, s>>>(cc);
+        else k_coarse_cycle<1, false><<<1, CC_THREADS, smem, s>>>(cc);
+        return;
+    }
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = cluster_config(smem, s, &attr);
+    if (y3) cudaLaunchKernelEx(&c, k_coarse_cycle<CC_CLUSTER, true>, cc);
+    else cudaLaunchKernelEx(&c, k_coarse_cycle<CC_CLUSTER, false>, cc);
 }
 void launch_coarse_inverse_many(const CoarseInv* items, const int* task, int ntask, cudaStream_t s) {
     if (ntask <= 0) return;

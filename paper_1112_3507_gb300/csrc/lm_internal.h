@@ -14,7 +14,6 @@ namespace lm {
 
 constexpr int COARSE_MAX = 16;      // coarsen while a level has more cells than this and an axis halves
 constexpr int COARSE_EXACT = 64;    // a coarsest level of at most this many cells is solved exactly
-constexpr int COARSE_SWEEPS = 32;   // (RB, BR) sweep pairs when it cannot be
 
 struct MgLevel {
     Lev32 L;
@@ -85,7 +84,11 @@ struct lm_grid {
     float* feat = nullptr;          // network input (N x 3)
     float* nny = nullptr;           // network output (N)
     std::vector<lm::MgLevel> mg;
-    int cc_level = -1;              // first level of the one-block coarse V-cycle (-1: none)
+    int cc_blocks = 1;              // blocks a coarse V-cycle's cluster may have
+    int cc_level = -1;              // first level of the one-launch coarse V-cycle (-1: none)
+    float4* cc_plan = nullptr;      // its plan (lm_coarse.cuh), formed again from every new hierarchy
+    bool plan_pending = false;      // hierarchy built, the plan not yet formed from it
+    int inverse_level = -1;         // first level smoothed with the correctly rounded inverse diagonal (-1: none)
     std::vector<double> history;
     // CUDA graphs of one inner flexible-CG iteration with the V-cycle (the
     // first and the later ones), captured on cap_stream for hierarchy
@@ -126,6 +129,13 @@ int net_set_params(lm_net* N, const float* host, int n);
 bool net_usable(const lm_grid* g);
 template <typename TV, typename TO>
 int net_apply(lm_grid* g, const TV* v, TO* dst, cudaStream_t s);
+// The first level the one-launch coarse V-cycle of at most nr_max blocks can
+// take over from (-1: none), and that cycle from level `lev` down: its solution
+// goes to x, its right-hand side is f.  inverse: g's inverse_level applies.
+int chain_level(const lm_grid* g, int nr_max);
+// plan: where the levels' plans lie (plan_size: its float4 count, or null).
+CoarseCycle coarse_chain(const lm_grid* g, int lev, int nr_max, bool inverse, float4* plan, float* x, const float* f,
+                         int nu1, int nu2, size_t* smem, size_t* plan_size = nullptr);
 Lev32 make_level(const int n[3], const int bc[3], const double h[3], const float* ct, const float* rho,
                  double rho_scale = 1.0);
 }  // namespace lm

@@ -134,37 +134,91 @@ void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const floa
                     int hy, int hz, const float* f, float* xout, int first, int zero, int prolong, int kz);
 void launch_resid_restrict(const Lev32& F, const Lev32& C, int hx, int hy, int hz, cudaStream_t s,
                            const float* x, const float* f, float* fc);
-// A whole coarse V-cycle (levels with at most CC_MAX_CELLS cells down to a
-// directly solved coarsest level) run by one block.
-constexpr int CC_MAXL = 5;
-constexpr int CC_MAX_CELLS = 4096;
+// A whole coarse V-cycle in one launch (lm_coarse.cuh): the levels of a chain
+// down to the coarsest, which is solved with its dense inverse or, when it has
+// none, by COARSE_SWEEPS sweep pairs.  A level of up to CC_MAX_PAIRS pairs of
+// x-neighbours (4096 cells with even rows; CC_PER pairs a thread is what its
+// registers hold) is run by one block, a larger one by the blocks of a cluster.
+constexpr int COARSE_SWEEPS = 32;                // (red-black, black-red) sweep pairs of an unsolved coarsest level
+constexpr int CC_MAXL = 8;
+constexpr int CC_THREADS = 512;                  // threads of a block that runs a cycle
+constexpr int CC_PER = 4;                        // pairs a thread owns on a chain level, at most
+constexpr int CC_MAX_PAIRS = CC_THREADS * CC_PER;
+constexpr int CC_PER_SHARED = 2;                 // ... on a level that the blocks of a cluster share
+constexpr int CC_CLUSTER = 16;                   // blocks of a cluster (the hardware's most)
+constexpr size_t CC_SMEM_MAX = 200 * 1024;       // shared-memory limit of a block
+// How a level's Gauss-Seidel values are formed: like the kernels that sweep
+// such a level on its own, weights face by face and an approximate division by
+// the diagonal (rbgs_tile) or one reciprocal for the two faces of an axis
+// (zrow2d_tile); or face by face with the correctly rounded inverse diagonal
+// (the levels of an exactly solved chain, see inverse_level).
+enum CCArith { CC_FACE, CC_AXIS, CC_INVERSE };
+struct CCLevel {
+    Lev32 L;
+    int hx, hy, hz;                // halvings to the next chain level
+    int nr;                        // blocks that share the level (never more than on the level before)
+    int arith;                     // CCArith
+    int hp, halo;                  // pairs a row; planes of halo each side (0: one block)
+    int npair, ncell, off;         // floats of an array by staged pair and by own cell; where the level's arrays lie
+    float ix, iy, iun, inr, imean; // 1 / nx, ny, units, nr, children of a cell of the next level
+    float4* plan;                  // the level's pairs as cc_plan_pair lays them out (not a solved coarsest level)
+};
 struct CoarseCycle {
-    int nl;                        // levels in the chain; the last is solved with ainv
-    Lev32 L[CC_MAXL];
-    int hx[CC_MAXL], hy[CC_MAXL], hz[CC_MAXL];   // halvings from chain level i to i + 1
-    float* x[CC_MAXL];             // level solutions (chain level 0: the caller's output)
-    float* f[CC_MAXL];             // level right-hand sides (chain level 0: the caller's rhs)
-    const float* ainv;
+    int nl;                        // levels in the chain
+    CCLevel lev[CC_MAXL];
+    int inv;                       // shared-memory offset (floats) of the dense inverse
+    int parts;                     // threads that share a row of it
+    float* x;                      // solution of chain level 0
+    const float* f;                // its right-hand side
+    const float* ainv;             // dense inverse of the coarsest level, or null
     int nu1, nu2;
 };
-constexpr int CC_THREADS = 1024;                 // threads of the block that runs a cycle
-constexpr int CC_PER = CC_MAX_CELLS / CC_THREADS;  // cells a thread owns on a chain level
-constexpr size_t CC_SMEM_MAX = 200 * 1024;       // shared-memory limit of the one-block cycle
-// Shared memory of the one-block cycle over levels of N_0 .. N_{nl-1} cells:
-// seven floats per cell and the dense inverse of the coarsest level.
-inline size_t cc_smem_bytes(const int* N, int nl) {
-    size_t b = 0;
-    for (int l = 0; l < nl; ++l) b += 7 * sizeof(float) * (size_t)N[l];
-    return b + sizeof(float) * (size_t)N[nl - 1] * (size_t)N[nl - 1];
+__host__ __device__ inline int cc_align4(int n) { return (n + 3) & ~3; }
+__host__ __device__ inline int cc_pairs(const Geo& g) { return ((g.nx + 1) >> 1) * g.ny * g.nz; }
+// A shared level is split into units of the planes that make one plane of the
+// next level; block r of nr owns the units from cc_unit0(r) to cc_unit0(r + 1).
+__host__ __device__ inline int cc_unit0(int r, int units, int nr) { return r * units / nr; }
+__host__ __device__ inline int cc_owner(int unit, int units, int nr) { return ((unit + 1) * nr - 1) / units; }
+// The most planes a block owns.
+__host__ __device__ inline int cc_own(const CCLevel& v) {
+    const int units = v.L.g.nz >> v.hz;
+    return ((units + v.nr - 1) / v.nr) << v.hz;
 }
-inline size_t cc_smem_bytes(const CoarseCycle& cc) {
-    int N[CC_MAXL];
-    for (int l = 0; l < cc.nl; ++l) N[l] = cc.L[l].g.N;
-    return cc_smem_bytes(N, cc.nl);
+// Fills the derived fields of the levels, lays a block's shared memory out
+// (per level the two colours of x by staged pair, right-hand side and residual
+// by own cell) and returns its bytes.
+inline size_t cc_layout(CoarseCycle& cc) {
+    size_t o = 0;
+    for (int l = 0; l < cc.nl; ++l) {
+        CCLevel& v = cc.lev[l];
+        const Geo& g = v.L.g;
+        v.hp = (g.nx + 1) >> 1;
+        v.halo = v.nr > 1 ? 1 : 0;
+        const int own = cc_own(v);
+        v.npair = cc_align4(v.hp * g.ny * (own + 2 * v.halo));
+        v.ncell = cc_align4(g.nx * g.ny * own);
+        v.off = (int)o;
+        v.ix = 1.f / (float)g.nx;
+        v.iy = 1.f / (float)g.ny;
+        v.iun = 1.f / (float)(g.nz >> v.hz);
+        v.inr = 1.f / (float)v.nr;
+        v.imean = 1.f / (float)((1 << v.hx) << v.hy << v.hz);
+        o += 2 * (size_t)v.npair + 2 * (size_t)v.ncell;
+    }
+    cc.inv = (int)o;
+    const size_t nc = (size_t)cc.lev[cc.nl - 1].L.g.N;
+    if (cc.ainv) o += nc * nc;
+    return sizeof(float) * o;
 }
-void launch_coarse_cycle(const CoarseCycle& cc, cudaStream_t s);
-void coarse_cycle_allow_smem();
-void rbgs_row_allow_smem();                      // raises the whole-row sweep's dynamic shared-memory limit                  // raises k_coarse_cycle's dynamic shared-memory limit
+constexpr int CC_PLAN = 6;                       // float4 arrays of a level's plan
+// forms the plan of cc's levels (cc.x, cc.f unused), or of `count` chains in device memory
+void launch_cc_plan(const CoarseCycle& cc, cudaStream_t s);
+void launch_cc_plan_many(const CoarseCycle* ccs, int count, cudaStream_t s);
+void launch_coarse_cycle(const CoarseCycle& cc, size_t smem, cudaStream_t s);
+// raises k_coarse_cycle's shared-memory and cluster-size limits; returns the
+// cluster size it can be launched with (1: no cluster)
+int coarse_cycle_allow();
+void rbgs_row_allow_smem();                      // raises the whole-row sweep's dynamic shared-memory limit
 void launch_coarse_inverse(const Lev32& L, cudaStream_t s, float* ainv);
 // one grid's coarsest level and where its dense inverse goes
 struct CoarseInv {
