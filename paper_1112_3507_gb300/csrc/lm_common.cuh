@@ -208,6 +208,13 @@ __device__ __forceinline__ void ff_add_prod(FF& s, float a, float b) {
     s.hi = t;
     s.lo = __fadd_rn(s.lo, __fadd_rn(e, pe));
 }
+__device__ __forceinline__ void ff_add(FF& s, float p) {
+    const float t = __fadd_rn(s.hi, p);
+    const float bp = __fsub_rn(t, s.hi);
+    const float e = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    s.hi = t;
+    s.lo = __fadd_rn(s.lo, e);
+}
 __device__ __forceinline__ double ff_value(const FF& s) { return (double)s.hi + (double)s.lo; }
 
 }  // namespace lm
