@@ -9,6 +9,8 @@
 // to threads with 2D/3D launches (no integer division per cell); the
 // stencils march along z keeping the z-neighbours in registers; and a whole
 // red-black sweep is one pass over memory (see rbgs_tile).
+#include <atomic>
+
 #include "lm_common.cuh"
 #include "lm_kernels.h"
 #include "lm_tiles.cuh"
@@ -2007,21 +2009,30 @@ int coarse_cycle_allow() {
     const void* const ks[] = {(const void*)k_coarse_cycle<1, false>, (const void*)k_coarse_cycle<1, true>,
                               (const void*)k_coarse_cycle<CC_CLUSTER, false>,
                               (const void*)k_coarse_cycle<CC_CLUSTER, true>};
-    int n = 0;
     for (int v = 0; v < 4; ++v) {
         cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM_MAX);
-        if (v < 2) continue;
-        cudaFuncSetAttribute(ks[v], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaLaunchAttribute attr;
-        const cudaLaunchConfig_t c = cluster_config(CC_SMEM_MAX, nullptr, &attr);
-        int m = 0;
-        if (cudaOccupancyMaxActiveClusters(&m, ks[v], &c) != cudaSuccess) {
-            cudaGetLastError();
-            m = 0;
-        }
-        n = v == 2 ? m : std::min(n, m);
+        if (v >= 2) cudaFuncSetAttribute(ks[v], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
-    return n > 0 ? CC_CLUSTER : 1;
+    // asked once per device: the question takes about half a millisecond
+    constexpr int MAX_DEV = 64;
+    static std::atomic<int> blocks[MAX_DEV];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return 1;
+    int n = blocks[dev].load();
+    if (n == 0) {
+        n = CC_CLUSTER;
+        for (int v = 2; v < 4; ++v) {
+            cudaLaunchAttribute attr;
+            const cudaLaunchConfig_t c = cluster_config(CC_SMEM_MAX, nullptr, &attr);
+            int m = 0;
+            if (cudaOccupancyMaxActiveClusters(&m, ks[v], &c) != cudaSuccess || m < 1) {
+                cudaGetLastError();
+                n = 1;
+            }
+        }
+        blocks[dev].store(n);
+    }
+    return n;
 }
 void launch_cc_plan(const CoarseCycle& cc, cudaStream_t s) {
     int pairs = 0;
