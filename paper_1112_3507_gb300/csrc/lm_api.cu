@@ -313,13 +313,25 @@ int solve_jacobi_pcg(lm_grid* g, const lm_solve_opts* o, lm_solve_result* res) {
     launch_pcg_init(a, g->G, s, o->use_x0 && g->have_x0);
     CK(cudaGetLastError());
     int k = 0, restarts = 0;
+    // small grids: up to 1024 iterations in one kernel, which stops by itself
+    // (a host check every check_every launches' worth would only slow it)
+    const bool run = g->coop && pcg_run_fits(g->N, g->G, g->nsm);
+    if (run && !g->bar && (rc = dalloc(&g->bar, 2))) return rc;
+    bool from_part = true;
     const int chunk = std::max(1, o->check_every);
     if ((rc = sync_state(g, g->st, s))) return rc;
     while (!g->st_host->done) {
-        for (int c = 0; c < chunk && k < o->max_iter; ++c, ++k) launch_pcg_iter(a, g->G, s, k);
+        if (run) {
+            const int k1 = (int)std::min<long long>(o->max_iter, (long long)k + 1024);
+            if ((rc = launch_pcg_run(a, g->G, g->nsm, s, k, k1, from_part, g->bar))) return rc;
+            from_part = false;
+        } else {
+            for (int c = 0; c < chunk && k < o->max_iter; ++c, ++k) launch_pcg_iter(a, g->G, s, k);
+        }
         CK(cudaGetLastError());
         if ((rc = sync_state(g, g->st, s))) return rc;
         SolveState* h = g->st_host;
+        if (run) k = h->iters;
         if (h->status) break;
         if (h->converged) {
             launch_true_residual(a, g->G, s);
@@ -328,6 +340,7 @@ int solve_jacobi_pcg(lm_grid* g, const lm_solve_opts* o, lm_solve_result* res) {
             ++restarts;
             k = g->st_host->iters;
             launch_pcg_restart(a, g->G, s, k);
+            from_part = true;
             if ((rc = sync_state(g, g->st, s))) return rc;
             continue;
         }
@@ -980,8 +993,11 @@ int lm_grid_create(int ndim, const int64_t n[3], const double h[3], const int bc
     // default 48 KB of shared memory: allow it before any entry point launches them
     rbgs_row_allow_smem();
     g->cc_blocks = coarse_cycle_allow();
-    int nsm = 1;
+    int nsm = 1, coop = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device);
+    g->nsm = nsm;
+    g->coop = coop != 0;
     const long long want = (N + NT - 1) / NT;
     g->G = (int)std::max(1LL, std::min<long long>(want, std::min<long long>(MAX_PARTIALS, (long long)nsm * 8)));
     g->geo = make_lev(g->n, g->bc, g->h, nullptr, nullptr).g;
@@ -1019,7 +1035,7 @@ void lm_grid_destroy(lm_grid* g) {
     free_mg(g);
     void* bufs[] = {g->ct, g->gx, g->gy, g->gz, g->dinv, g->f, g->x, g->x0, g->r, g->p, g->q,
                     g->ct32, g->rho32, g->r32, g->e32, g->z32, g->p32, g->q32, g->tmp_a, g->tmp_b,
-                    g->scal, g->ctr, g->stage, g->part,
+                    g->scal, g->ctr, g->bar, g->stage, g->part,
                     g->dscal, g->st, g->st_in, g->hist_dev, g->asm_fl};
     for (void* b : bufs) cudaFree(b);
     cudaFreeHost(g->st_host);

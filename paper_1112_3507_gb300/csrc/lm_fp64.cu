@@ -7,6 +7,8 @@
 // per cell minimal (face conductances and the inverse Jacobi diagonal are
 // computed once, at assembly; the stencil uses 13 float64 operations per 3D
 // cell) and stream each vector once per kernel.
+#include <algorithm>
+
 #include "lm_common.cuh"
 #include "lm_kernels.h"
 #include "lm_tiles.cuh"
@@ -184,6 +186,279 @@ __global__ void __launch_bounds__(NT) k_pcg_p(PcgArgs a, int k) {
     const int stride = gridDim.x * blockDim.x;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < a.g.N; idx += stride)
         a.p[idx] = a.op.dinv[idx] * a.r[idx] + beta * a.p[idx];
+}
+
+// ---- the same iterations in one cooperative kernel ------------------------------
+//
+// On a grid of a few hundred thousand cells an iteration's three launches cost
+// more than its arithmetic (24 us an iteration on 129 x 97 cells, of which
+// 0.5 us float64 work), so k_pcg_run runs iterations k0, k0 + 1, ... until the
+// solve is done, or k1, without leaving the GPU.  One block per SM keeps its
+// cells' x, r, p, q (and, with at most four cells a thread, the operator's
+// coefficients) in registers; only p, which neighbours read, and the block
+// sums go through L2.  Three grid barriers an iteration stand where the
+// launches ended, one thread a block looking at one counter.  (Sums tagged
+// with their iteration and waited for by every thread that adds them, in place
+// of two of the barriers, took 34 us an iteration: the looks crowd out the
+// stores they wait for.)
+//
+// Every sum is formed in the order of k_pcg_apply, k_pcg_xr and k_pcg_p
+// launched with G blocks (one cell a thread: G = ceil(N / 256)), so the
+// iterates are bitwise theirs.  With fewer than one such block per SM its
+// warps are dealt out over the SMs (WARPS: sums are kept per warp and added as
+// block_sum adds them), because one SM's float64 pipe takes 18 cycles an
+// instruction; otherwise block b takes the blocks b, b + gridDim.x, ...
+//
+// Every wait is bounded: past the limit the waiting block raises the error
+// flag, which every block sees at its next look, and all return
+// (LM_ERR_TIMEOUT).
+//
+// 129 x 97 cells: 22.9 -> 11.2 us an iteration, 59 x 17 x 65: 31.1 -> 14.8 us,
+// 81 x 49 x 70: 86.4 -> 35.9 us.  What is left on the small grids is latency:
+// three round trips to L2, three barriers and a chain of some forty dependent
+// float64 steps (operator, sums, quotients).
+constexpr unsigned BAR_LIMIT = 1u << 22;            // looks of about 1 us
+
+// bar[0]: arrivals since the launch; bar[1]: a block gave up.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& target) {
+    __shared__ int s_ok;
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        int ok = 0;
+        for (unsigned n = 0; n < BAR_LIMIT; ++n) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= target) {
+                ok = 1;
+                break;
+            }
+            if ((n & 255) == 255 && *(volatile unsigned*)(bar + 1)) break;
+        }
+        if (!ok) atomicExch(bar + 1, 1u);
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// block_sum<Q> of a block of NT threads, the result in thread 0: warps that hold
+// only zeros (any = false) and the steps of the last tree that would add zeros
+// are left out, which changes no sum.
+template <int Q>
+__device__ __forceinline__ void pcg_block_sum(double (&v)[Q], bool any, double* smem) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (any)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if (l == 0)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) smem[q * 32 + w] = v[q];
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] = l < NT / 32 ? smem[q * 32 + l] : 0.0;
+#pragma unroll
+        for (int o = NT / 64; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    }
+    __syncthreads();
+}
+
+// Sums of the G block partials of the slots (WARPS: of the 8 G warp partials,
+// eight a block, added as block_sum's last tree adds them) in the order of
+// reduce_partials; the result in thread 0.
+template <bool WARPS, int Q>
+__device__ __forceinline__ void pcg_totals(const double* part, const int (&slot)[Q], int G, double* smem,
+                                           double (&v)[Q]) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const double* const p = part + slot[q] * MAX_PARTIALS;
+        v[q] = 0.0;
+        for (int t = threadIdx.x; t < G; t += NT) {
+            if constexpr (WARPS) {
+                double w[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) w[u] = __ldcg(p + 8 * t + u);
+                v[q] += ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+            } else {
+                v[q] += __ldcg(p + t);
+            }
+        }
+    }
+    pcg_block_sum<Q>(v, (int)(threadIdx.x & ~31u) < G, smem);
+}
+// The thread's values v of unit u (virtual block, or warp) into the slots of part.
+template <bool WARPS, int Q>
+__device__ __forceinline__ void pcg_partial(double (&v)[Q], int u, double* part, const int (&slot)[Q], double* smem) {
+    if constexpr (!WARPS) {
+        pcg_block_sum<Q>(v, true, smem);
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    }
+    if (WARPS ? (threadIdx.x & 31) == 0 : threadIdx.x == 0)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) part[slot[q] * MAX_PARTIALS + u] = v[q];
+}
+
+template <bool WARPS, int K>
+__global__ void __launch_bounds__(NT, 1) k_pcg_run(PcgArgs a, int G, int k0, int k1, int from_part,
+                                                   unsigned* __restrict__ bar) {
+    constexpr bool KEEP = K <= 4;                   // coefficients in registers
+    __shared__ double sm[64];
+    // scalars of an iteration: formed by one thread each, since every warp that
+    // repeats a division occupies the float64 pipe for it
+    __shared__ double s_rr, s_rz, s_alpha, s_beta;
+    __shared__ int s_bad, s_stop;
+    const Geo& g = a.g;
+    const int tid = threadIdx.x, units = WARPS ? 8 * G : G;
+    const int u0 = WARPS ? (int)(blockIdx.x + gridDim.x * (tid >> 5)) : (int)blockIdx.x;
+    unsigned target = 0;
+    // the thread's cells: index (-1: none), neighbours, coefficients, vectors
+    int id[K], xm[K], xp[K], ym[K], yp[K], zm[K], zp[K];
+    double c[K], wxm[K], wxp[K], wym[K], wyp[K], wzm[K], wzp[K], di[K], x[K], r[K], p[K], q[K];
+#pragma unroll
+    for (int n = 0; n < K; ++n) {
+        const int u = u0 + n * gridDim.x, idx = u < units ? (WARPS ? 32 * u + (tid & 31) : NT * u + tid) : g.N;
+        id[n] = idx < g.N ? idx : -1;
+        x[n] = r[n] = p[n] = q[n] = 0.0;
+        if (id[n] < 0) continue;
+        int i, j, k;
+        cell_coords(idx, g, i, j, k);
+        Nbr nb = nbr_x(idx, i, g);
+        xm[n] = nb.im, xp[n] = nb.ip;
+        nb = nbr_y(idx, j, g);
+        ym[n] = nb.im, yp[n] = nb.ip;
+        nb = nbr_z(idx, k, g);
+        zm[n] = nb.im, zp[n] = nb.ip;
+        if (KEEP) {
+            c[n] = a.op.ct[idx], di[n] = a.op.dinv[idx];
+            wxm[n] = a.op.gx[idx], wxp[n] = a.op.gx[xp[n]];
+            wym[n] = a.op.gy[idx], wyp[n] = a.op.gy[yp[n]];
+            wzm[n] = a.op.gz[idx], wzp[n] = a.op.gz[zp[n]];
+        }
+        x[n] = a.x[idx], r[n] = a.r[idx], p[n] = a.p[idx];
+    }
+    double rz = from_part ? reduce_partials(a.part + (2 + (k0 & 1)) * MAX_PARTIALS, G, sm) : a.st->scale;
+    const double fnorm = a.st->fnorm, rtol = a.st->rtol;
+    bool ok = true;
+    for (int k = k0; k < k1; ++k) {
+        // q = A p, p.q
+#pragma unroll
+        for (int n = 0; n < K; ++n) {
+            const int u = u0 + n * gridDim.x;
+            if (u >= units) break;
+            double acc[1] = {0.0};
+            if (id[n] >= 0) {
+                const int idx = id[n];
+                const double pc = p[n];
+                double y = (KEEP ? c[n] : a.op.ct[idx]) * pc;
+                y += (KEEP ? wxm[n] : a.op.gx[idx]) * (pc - __ldcg(a.p + xm[n]));
+                y += (KEEP ? wxp[n] : a.op.gx[xp[n]]) * (pc - __ldcg(a.p + xp[n]));
+                if (g.ny > 1) {
+                    y += (KEEP ? wym[n] : a.op.gy[idx]) * (pc - __ldcg(a.p + ym[n]));
+                    y += (KEEP ? wyp[n] : a.op.gy[yp[n]]) * (pc - __ldcg(a.p + yp[n]));
+                }
+                y += (KEEP ? wzm[n] : a.op.gz[idx]) * (pc - __ldcg(a.p + zm[n]));
+                y += (KEEP ? wzp[n] : a.op.gz[zp[n]]) * (pc - __ldcg(a.p + zp[n]));
+                q[n] = y;
+                acc[0] += pc * y;
+            }
+            const int sl[1] = {0};
+            pcg_partial<WARPS, 1>(acc, u, a.part, sl, sm);
+        }
+        if (!(ok = grid_barrier(bar, target))) break;
+        // alpha, x, r, r.r, r.z
+        {
+            const int sl[1] = {0};
+            double pq[1];
+            pcg_totals<WARPS, 1>(a.part, sl, G, sm, pq);
+            if (tid == 0) {
+                s_bad = !(pq[0] > 0.0) || !isfinite(pq[0]) || !isfinite(rz);
+                s_alpha = rz / pq[0];
+            }
+            __syncthreads();
+        }
+        if (s_bad) {                                 // the same verdict in every block
+            if (blockIdx.x == 0 && tid == 0) {
+                a.st->status = LM_ERR_BREAKDOWN;
+                a.st->done = 1;
+            }
+            break;
+        }
+        const double alpha = s_alpha;
+#pragma unroll
+        for (int n = 0; n < K; ++n) {
+            const int u = u0 + n * gridDim.x;
+            if (u >= units) break;
+            double acc[2] = {0.0, 0.0};
+            if (id[n] >= 0) {
+                x[n] += alpha * p[n];
+                const double ri = r[n] - alpha * q[n];
+                r[n] = ri;
+                acc[0] += ri * ri;
+                acc[1] += ri * ((KEEP ? di[n] : a.op.dinv[id[n]]) * ri);
+            }
+            const int sl[2] = {1, 2 + ((k + 1) & 1)};
+            pcg_partial<WARPS, 2>(acc, u, a.part, sl, sm);
+        }
+        if (!(ok = grid_barrier(bar, target))) break;
+        // beta, p; the convergence test is formed meanwhile and looked at after
+        // the barrier (a p updated past the end is not used)
+        {
+            const int sl[2] = {1, 2 + ((k + 1) & 1)};
+            double t[2];
+            pcg_totals<WARPS, 2>(a.part, sl, G, sm, t);
+            if (tid == 0) {
+                s_rr = t[0];
+                s_rz = t[1];
+            }
+            __syncthreads();
+            if (tid == 32) s_beta = s_rz / rz;
+            __syncthreads();
+        }
+        const double rz_new = s_rz, beta = s_beta;
+#pragma unroll
+        for (int n = 0; n < K; ++n)
+            if (id[n] >= 0) {
+                p[n] = (KEEP ? di[n] : a.op.dinv[id[n]]) * r[n] + beta * p[n];
+                __stcg(a.p + id[n], p[n]);
+            }
+        if (tid == NT - 1) {
+            const double rel = sqrt(s_rr) / fnorm;
+            const bool conv = rel <= rtol, bad = !isfinite(rel) || !isfinite(rz_new) || !(rz != 0.0);
+            s_stop = conv || bad || k + 1 >= a.max_iter;
+            if (blockIdx.x == 0) {
+                a.hist[k + 1] = rel;
+                a.st->iters = k + 1;
+                a.st->rel = rel;
+                a.st->scale = rz_new;
+                if (conv) a.st->converged = 1;
+                if (bad) a.st->status = LM_ERR_BREAKDOWN;
+                if (s_stop) a.st->done = 1;
+            }
+        }
+        rz = rz_new;
+        if (!(ok = grid_barrier(bar, target)) || s_stop) break;
+    }
+    if (!ok && tid == 0) {
+        a.st->status = LM_ERR_TIMEOUT;
+        a.st->done = 1;
+    }
+#pragma unroll
+    for (int n = 0; n < K; ++n)
+        if (id[n] >= 0) {
+            a.x[id[n]] = x[n];
+            a.r[id[n]] = r[n];
+            a.q[id[n]] = q[n];
+        }
 }
 
 // r = f - A x, partial r.r (slot 1): the true residual
@@ -452,6 +727,26 @@ void launch_pcg_iter(const PcgArgs& a, int G, cudaStream_t s, int k) {
     k_pcg_xr<<<G, NT, 0, s>>>(a, k);
     count_launches(1);
     k_pcg_p<<<G, NT, 0, s>>>(a, k);
+}
+// The line lies where the kernel's registers end: eight cells a thread of one
+// block per SM (311,296 cells on 152 SMs), which is also where a launch's
+// blocks stop having one cell a thread.  Larger grids are bound by the float64
+// pipe, not by the launches.
+bool pcg_run_fits(int N, int G, int nsm) { return (long long)G * NT >= N && G <= 8 * nsm ; }
+int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int k1, int from_part, unsigned* bar) {
+    if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return LM_ERR_CUDA;
+    const void* f;
+    int blocks = nsm;
+    if (G < nsm) {
+        f = (const void*)k_pcg_run<true, 1>;
+        blocks = std::min(nsm, 2 * G);               // four warps with cells a block: 11.2 us, one or two: 12.3
+    } else if (G <= 2 * nsm) f = (const void*)k_pcg_run<false, 2>;
+    else if (G <= 4 * nsm) f = (const void*)k_pcg_run<false, 4>;
+    else f = (const void*)k_pcg_run<false, 8>;
+    PcgArgs args = a;
+    void* av[] = {&args, &G, &k0, &k1, &from_part, &bar};
+    count_launches(1);
+    return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(NT), av, 0, s) == cudaSuccess ? LM_OK : LM_ERR_CUDA;
 }
 void launch_true_residual(const PcgArgs& a, int G, cudaStream_t s) {
     count_launches(1);

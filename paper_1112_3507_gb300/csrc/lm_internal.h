@@ -52,6 +52,9 @@ struct lm_grid {
     float *tmp_a = nullptr, *tmp_b = nullptr;   // level-0 sweep buffers
     double* scal = nullptr;         // reduction results (float32 kernels)
     unsigned int* ctr = nullptr;    // last-block arrival counter
+    unsigned int* bar = nullptr;    // grid barrier of the cooperative Jacobi-PCG kernel (on first use)
+    int nsm = 1;                    // SMs of the device
+    bool coop = false;              // cooperative launches are available
     double* stage = nullptr;        // 3N host-input staging (allocated on first use)
     // host inputs of an assembly arrive in chunks of planes on copy_stream
     // (one event per chunk) while the assembly of the chunks before runs
