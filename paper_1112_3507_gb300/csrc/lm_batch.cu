@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(NT) kb_ir_residual(const BTask* __restrict__ T
     for (int idx = t.lblk * NT + threadIdx.x; idx < G.N; idx += stride) {
         const double fi = G.f[idx];
         const double ri = zero_x ? fi : fi - apply64_at(idx, G.geo, G.op, G.x);
-        G.r32[idx] = (float)ri;
+        G.r32[idx] = to_f32(ri);
         acc[0] += ri * ri;
         if (first) acc[1] += fi * fi;                 // ||f|| is kept from the first residual
     }
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(NT) kb_ir_correct(const BTask* __restrict__ T,
     const BGrid& G = Gs[t.g];
     if (G.st->done) return;
     const int stride = t.nblk * NT;
-    for (int idx = t.lblk * NT + threadIdx.x; idx < G.N; idx += stride) G.x[idx] += (double)G.e32[idx];
+    for (int idx = t.lblk * NT + threadIdx.x; idx < G.N; idx += stride) G.x[idx] += to_f64(G.e32[idx]);
 }
 
 // out[g] = the outer state, out[count + g] = the inner state

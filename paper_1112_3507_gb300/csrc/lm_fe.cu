@@ -201,8 +201,12 @@ struct FeFlags {
     int bad32;     // a float32 coefficient outside the normal float32 range
 };
 
-__device__ __forceinline__ bool pos_finite(double v) { return v > 0.0 && v < INFINITY; }
-__device__ __forceinline__ bool normal32(double v) { return v == 0.0 || (fabs(v) < 0x1p126 && fabs(v) > 0x1p-125); }
+using lm::pos_finite;
+// 0, or 2^-125 < |v| < 2^126, by the bits
+__device__ __forceinline__ bool normal32(double v) {
+    const uint64_t m = (uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return m == 0 || (m > (898ull << 52) && m < (1149ull << 52));
+}
 
 // kappa_e of the element with lowest corner idx (0 past a wall) and V c~.
 __global__ void __launch_bounds__(NT) k_fe_setup(FeGeo g, const double* __restrict__ ct,
@@ -231,7 +235,7 @@ __global__ void __launch_bounds__(NT) k_fe_setup(FeGeo g, const double* __restri
                         s += rho[zs[c] + ys[b] + xs[a]];
                         ++cnt;
                     }
-            e = cnt / s;
+            e = lm::idiv((double)cnt, s);
         }
         ke[idx] = e;
         vc[idx] = vol1(i, g.nx, g.wx, g.hx) * vol1(j, g.ny, g.wy, g.hy) * vol1(k, g.nz, g.wz, g.hz) * cti;
@@ -258,13 +262,13 @@ __global__ void __launch_bounds__(NT) k_fe_diag(FeGeo g, double kd, const double
             for (int b = 0; b < ny2; ++b)
                 for (int a = 0; a < 2; ++a) s += ke[zs[c] + ys[b] + xs[a]];
         const double d = vc[idx] + kd * s;
-        const double di = 1.0 / d;
+        const double di = lm::ircp(d);
         dinv[idx] = di;
         const double kei = ke[idx], vci = vc[idx];
         bad32 |= !normal32(kei) || !normal32(vci) || !normal32(di);
-        ke32[idx] = (float)kei;
-        vc32[idx] = (float)vci;
-        dinv32[idx] = (float)di;
+        ke32[idx] = lm::to_f32(kei);
+        vc32[idx] = lm::to_f32(vci);
+        dinv32[idx] = lm::to_f32(di);
     }
     if (bad32) atomicOr(&fl->bad32, 1);
 }
@@ -274,7 +278,7 @@ __global__ void __launch_bounds__(NT) k_fe_ctilde(int N, double dt, const double
                                                   double* out) {
     const double dt2 = dt * dt;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x)
-        out[idx] = 1.0 / ((dt2 * rho_old[idx]) * cs2[idx]);
+        out[idx] = lm::ircp((dt2 * rho_old[idx]) * cs2[idx]);
 }
 
 // b = V f (f may alias b)
@@ -339,8 +343,8 @@ __global__ void __launch_bounds__(NT) k_fe_resid64(FeOp<double> op, const double
 // the last block sets st->rel = ||r|| / ||f|| (and st->fnorm when SET_FNORM).
 template <bool SET_FNORM>
 __global__ void __launch_bounds__(NT) k_fe_ir_res64(FeOp<double> op, const double* __restrict__ f, double* x,
-                                                    float* __restrict__ r32, int zero_x, double rscale, Red red,
-                                                    SolveState* st) {
+                                                    float* __restrict__ r32, int zero_x, double rscale, int kscale,
+                                                    Red red, SolveState* st) {
     __shared__ double sm[64];
     double acc[2] = {0.0, 0.0};
     auto ld = [&](int j) { return x[j]; };
@@ -349,9 +353,9 @@ __global__ void __launch_bounds__(NT) k_fe_ir_res64(FeOp<double> op, const doubl
         double xc;
         const double ri = zero_x ? fi : fi - bx_point(idx, op, ld, xc);
         if (zero_x) x[idx] = 0.0;
-        r32[idx] = (float)(ri * rscale);
+        r32[idx] = lm::to_f32(lm::mul_pow2(ri, rscale, kscale));
         acc[0] += ri * ri;
-        acc[1] += fi * fi;
+        if (SET_FNORM) acc[1] += fi * fi;             // ||f|| is kept from the first residual
     }
     const int sl[2] = {SLOT_RR, SLOT_FF};
     if (lm::grid_reduce<2>(acc, red, sl, sm) && threadIdx.x == 0) {
@@ -682,9 +686,11 @@ void launch_fe_ir_res(const lm_fe* fe, cudaStream_t s, int zero_x, int set_fnorm
     lm::count_launches(1);
     const FeOp<double> op = fe_op<double>(fe);
     if (set_fnorm)
-        k_fe_ir_res64<true><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, fe_red(fe), fe->st);
+        k_fe_ir_res64<true><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, lm::pow2_of(rscale),
+                                                      fe_red(fe), fe->st);
     else
-        k_fe_ir_res64<false><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, fe_red(fe), fe->st);
+        k_fe_ir_res64<false><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, lm::pow2_of(rscale),
+                                                      fe_red(fe), fe->st);
 }
 
 lm::PcgArgs fe_pcg_args(lm_fe* fe, int max_iter) {

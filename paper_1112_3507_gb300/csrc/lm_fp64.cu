@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(NT) k_jacobi_diag(Geo g, const double* __restr
         cell_coords(idx, g, i, j, k);
         const double d = ct[idx] + gx[idx] + gx[nbr_x(idx, i, g).ip] + gy[idx] + gy[nbr_y(idx, j, g).ip] +
                          gz[idx] + gz[nbr_z(idx, k, g).ip];
-        dinv[idx] = 1.0 / d;
+        dinv[idx] = ircp(d);
     }
 }
 
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(NT) k_ir_residual(Geo g, Op64 op, const double
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx += stride) {
         const double fi = f[idx];
         const double ri = zero_x ? fi : fi - apply64_at(idx, g, op, x);
-        r32[idx] = SC == 2 ? (float)(ri * rscale) : (SC == 1 ? (float)ri * rs32 : (float)ri);
+        r32[idx] = SC == 2 ? (float)(ri * rscale) : (SC == 1 ? to_f32(ri) * rs32 : to_f32(ri));
         acc[0] += ri * ri;
         if (FNORM) acc[1] += fi * fi;
     }
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(NT) k_ir_correct(int N, double* __restrict__ x
                                                    double escale) {
     const int stride = gridDim.x * blockDim.x;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += stride)
-        x[idx] += (double)e[idx] * escale;
+        x[idx] += to_f64(e[idx]) * escale;
 }
 
 

@@ -86,8 +86,8 @@ __global__ void __launch_bounds__(lm::NT) k_advect(AdvGeo G, AdvIO io, double dt
             // the five, plus face between 2 and 3
             const double* rho = io.q[0];
             const double* m = io.q[1 + a];
-            const double um = wall_m ? 0.0 : (m[id[1]] + m[id[2]]) / (rho[id[1]] + rho[id[2]]);
-            const double up = wall_p ? 0.0 : (m[id[2]] + m[id[3]]) / (rho[id[2]] + rho[id[3]]);
+            const double um = wall_m ? 0.0 : lm::idiv(m[id[1]] + m[id[2]], rho[id[1]] + rho[id[2]]);
+            const double up = wall_p ? 0.0 : lm::idiv(m[id[2]] + m[id[3]], rho[id[2]] + rho[id[3]]);
             for (int q = 0; q < G.nq; ++q) {
                 const double* v = io.q[q];
                 double x[5];
@@ -113,10 +113,10 @@ __global__ void __launch_bounds__(lm::NT) k_eos_ideal(int N, double gamma, const
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x) {
         const double r = rho[idx];
         const double mx = mom[idx], my = mom[(size_t)N + idx], mz = mom[2 * (size_t)N + idx];
-        const double kin = 0.5 * (mx * mx + my * my + mz * mz) / r;
+        const double kin = lm::idiv(0.5 * (mx * mx + my * my + mz * mz), r);
         const double pi = (gamma - 1.0) * (e[idx] - kin);
         p[idx] = pi;
-        if (cs2) cs2[idx] = gamma * pi / r;
+        if (cs2) cs2[idx] = lm::idiv(gamma * pi, r);
     }
 }
 

@@ -1,0 +1,150 @@
+// Float64 operations on the integer pipe, bit for bit those of the float64 one.
+//
+// GB300 issues float64 at 1/74 of the float32 rate -- comparisons and
+// conversions included -- so in a kernel bound by the float64 pipe every such
+// instruction that a few integer instructions can stand for is better done by
+// them.
+//
+// Quotients.  A float64 quotient is a dozen dependent float64 instructions, and
+// the kernels that form face conductances, face velocities and pressures spent
+// most of their float64 time on divisions.  With both mantissas as 53-bit
+// integers A and B:
+//
+//   y0 = 24 bits of 1/B from the float32 reciprocal approximation of B's
+//        leading 24 bits,
+//   y  = y0 (1 + e + e^2), e = 1 - B y0 exactly: Newton's series for the
+//        reciprocal to third order, 60 bits in fixed point,
+//   Q  = A y truncated, biased down so that it is the quotient's integer part or
+//        one less,
+//   and the exact remainder A 2^s - Q B (mod 2^64, since it fits) rounds it.
+//
+// A quotient of two 53-bit integers is never halfway between two 53-bit
+// results, so the remainder's comparison with B / 2 is the rounding to nearest
+// (Markstein's and every remainder-based division's last step): the bits are
+// those of the hardware's a / b and __drcp_rn, checked exhaustively at the
+// mantissas' corners and on random pairs.  Operands or results outside the
+// normal range (subnormals, infinities, NaN, a zero divisor) take the
+// hardware's path; a zero dividend, common in fields at rest, is a zero.
+//
+// About 65 integer instructions, against seven (reciprocal) and eleven
+// (quotient) issue slots of the float64 pipe at 18.5 cycles an SM each.
+//
+// Sign, finiteness and order of float64 values are those of their bits; a
+// conversion between normal float32 and float64 values shifts the mantissa.
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define LM_HD __host__ __device__ __forceinline__
+#else
+#define LM_HD inline
+#endif
+
+namespace lm {
+
+// 2^63 / m for m = B / 2^52 in [1, 2), off by less than 2^4, from the bits of
+// y0 in [1/2, 1], off from 1 / m by less than 2^-21.
+LM_HD uint64_t idiv_recip(uint64_t B, uint32_t y0_bits) {
+    // y0 as an integer at scale 2^24
+    const uint32_t Y0 = ((y0_bits & 0x7fffffu) | 0x800000u) << ((y0_bits >> 23) - 126u);
+    const uint64_t P = (uint64_t)(uint32_t)B * Y0 + ((uint64_t)((uint32_t)(B >> 32) * Y0) << 32);
+    const int64_t E = -(int64_t)P;                             // (1 - m y0) 2^76, |E| < 2^55
+    const int32_t eh = (int32_t)(E >> 24);
+    const int64_t F = E + (((int64_t)eh * eh) >> 28);          // (e + e^2) 2^76
+    const int64_t T = ((int64_t)(int32_t)Y0 * (int32_t)(F >> 32) + (int64_t)(((uint64_t)Y0 * (uint32_t)F) >> 32)) >> 5;
+    return ((uint64_t)Y0 << 39) + (uint64_t)T;
+}
+
+LM_HD uint64_t idiv_mulhi(uint64_t a, uint64_t b) {
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (uint64_t)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+
+// Mantissa and exponent of the rounded quotient of normal operands as one
+// integer: e 2^52 + Q - 2^52 (Q = 2^53 carries into the exponent); e is the
+// biased exponent, valid when 1 <= e <= 2046 before and after.
+LM_HD int64_t idiv_core(uint64_t ma, uint64_t mb, int e, uint64_t y) {
+    const uint64_t A = ma | (1ull << 52), B = mb | (1ull << 52);
+    const int less = A < B;                                    // quotient in (1/2, 1): one more bit
+    const uint64_t q62 = idiv_mulhi(A << 11, y) - 16;          // A / B at scale 2^62, low by less than 2^6
+    uint64_t Q = q62 >> (10 - less);
+    const int64_t rem2 = 2 * (int64_t)((A << (52 + less)) - Q * B);   // twice the remainder, in [0, 4 B)
+    Q += (rem2 > (int64_t)B) + (rem2 > (int64_t)(3 * B));
+    return ((int64_t)(e - less) << 52) + (int64_t)(Q - (1ull << 52));
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ uint32_t idiv_seed(uint64_t m) {
+    const float f = __uint_as_float(0x3f800000u | (uint32_t)(m >> 29));
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+    return __float_as_uint(fmaxf(r, 0.5f));
+}
+
+// a / b, rounded to nearest
+__device__ __forceinline__ double idiv(double a, double b) {
+    const uint64_t ua = (uint64_t)__double_as_longlong(a), ub = (uint64_t)__double_as_longlong(b);
+    const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff, e = ea - eb + 1023;
+    const uint64_t M = (1ull << 52) - 1;
+    // normal operands and a result that stays normal whichever way it rounds
+    if ((unsigned)(ea - 1) < 2046u && (unsigned)(eb - 1) < 2046u && (unsigned)(e - 2) < 2044u) {
+        const uint64_t mb = ub & M;
+        const int64_t r = idiv_core(ua & M, mb, e, idiv_recip(mb | (1ull << 52), idiv_seed(mb)));
+        return __longlong_as_double(r | (int64_t)((ua ^ ub) & (1ull << 63)));
+    }
+    if (!(ua << 1) && (unsigned)(eb - 1) < 2046u) return __longlong_as_double((long long)((ua ^ ub) & (1ull << 63)));
+    return a / b;
+}
+// 1 / b, rounded to nearest
+__device__ __forceinline__ double ircp(double b) { return idiv(1.0, b); }
+
+// v > 0 and finite
+__device__ __forceinline__ bool pos_finite(double v) {
+    return (uint64_t)(__double_as_longlong(v) - 1) < 0x7ff0000000000000ull - 1;
+}
+
+// (float)v, rounded to nearest even
+__device__ __forceinline__ float to_f32(double v) {
+    const uint64_t u = (uint64_t)__double_as_longlong(v), m = u & 0x7fffffffffffffffull;
+    // exponents of normal float32 values, one short of the largest so that a
+    // carry is one too
+    if (m - (897ull << 52) < (1149ull - 897ull + 1) << 52) {
+        const uint32_t r = (uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29) - (896u << 23);
+        return __uint_as_float(r | (uint32_t)(u >> 32 & 0x80000000u));
+    }
+    if (!m) return __uint_as_float((uint32_t)(u >> 32));
+    return (float)v;
+}
+// (double)v
+__device__ __forceinline__ double to_f64(float v) {
+    const uint32_t u = __float_as_uint(v), e = u >> 23 & 255u;
+    if (e - 1u < 254u)
+        return __longlong_as_double((long long)((((uint64_t)(u & 0x7fffffffu) << 29) + (896ull << 52)) |
+                                                ((uint64_t)(u & 0x80000000u) << 32)));
+    if (!(u << 1)) return __longlong_as_double((long long)((uint64_t)u << 32));
+    return (double)v;
+}
+
+// v times a factor that is 2^k, or no such power (k = POW2_NONE)
+constexpr int POW2_NONE = 0x7fffffff;
+__device__ __forceinline__ double mul_pow2(double v, double factor, int k) {
+    const uint64_t u = (uint64_t)__double_as_longlong(v);
+    const int e = (int)(u >> 52) & 0x7ff;
+    if (k != POW2_NONE && (unsigned)(e - 1) < 2046u && (unsigned)(e + k - 1) < 2046u)
+        return __longlong_as_double((long long)u + ((long long)k << 52));
+    if (!(u << 1) && k != POW2_NONE) return v;
+    return v * factor;
+}
+#endif
+// the exponent k of a factor 2^k, else POW2_NONE (host)
+inline int pow2_of(double f) {
+    int e = 0;
+    return f > 0.0 && f < 1e300 && frexp(f, &e) == 0.5 && e > -1000 && e < 1000 ? e - 1 : 0x7fffffff;
+}
+
+}  // namespace lm

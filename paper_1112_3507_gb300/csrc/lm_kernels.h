@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "lm_common.cuh"
+#include "lm_intfp.cuh"
 
 namespace lm {
 
@@ -70,12 +71,14 @@ struct AsmArgs {
     double dt;
     int raw;
     double c2x, c2y, c2z;    // 2 / h^2 per axis
+    int kx, ky, kz;          // their exponents where they are powers of two (pow2_of)
     Op64Out out;
     AsmFlags* fl;
 };
 inline AsmArgs asm_args(const Geo& g, const double* a_in, const double* rho_new, const double* cs2, double dt,
                         int raw, const double h[3], const Op64Out& out, AsmFlags* fl) {
-    return AsmArgs{g, a_in, rho_new, cs2, dt, raw, 2.0 / (h[0] * h[0]), 2.0 / (h[1] * h[1]), 2.0 / (h[2] * h[2]),
+    const double c[3] = {2.0 / (h[0] * h[0]), 2.0 / (h[1] * h[1]), 2.0 / (h[2] * h[2])};
+    return AsmArgs{g,    a_in, rho_new, cs2, dt, raw, c[0], c[1], c[2], pow2_of(c[0]), pow2_of(c[1]), pow2_of(c[2]),
                    out, fl};
 }
 

@@ -48,17 +48,17 @@ __device__ __forceinline__ void assemble_range(const AsmArgs& a, int start, int 
     for (int idx = start; idx < stop; idx += stride) {
         const double rn = rho_new[idx];
         double c;
-        bool ok = rn > 0.0 && isfinite(rn);
+        bool ok = pos_finite(rn);
         if (raw) {
             c = a_in[idx];
         } else {
             const double ro = a_in[idx], c2 = cs2[idx];
-            ok = ok && ro > 0.0 && isfinite(ro) && c2 > 0.0 && isfinite(c2);
-            c = __drcp_rn((dt * dt) * ro * c2);                // Eq. cpoiss: 1/(...) rounded to nearest
+            ok = ok && pos_finite(ro) && pos_finite(c2);
+            c = ircp((dt * dt) * ro * c2);                     // Eq. cpoiss: 1/(...) rounded to nearest
         }
-        ok = ok && c > 0.0 && isfinite(c);
+        ok = ok && pos_finite(c);
         if (!ok) atomicOr(&fl->bad, 1);
-        if (rn > 0.0 && isfinite(rn)) {
+        if (pos_finite(rn)) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(rn);
             rmax = b > rmax ? b : rmax;
             rmin = b < rmin ? b : rmin;
@@ -66,21 +66,26 @@ __device__ __forceinline__ void assemble_range(const AsmArgs& a, int start, int 
         int i, j, k;
         cell_coords(idx, g, i, j, k);
         // g_f = kappa_f / h^2 with kappa_f = 2/(rho_L + rho_R) (Eq. kappapoiss, harmonic
-        // mean), evaluated as (2/h^2) * RN(1/(rho_L + rho_R)): a correctly rounded
-        // float64 reciprocal per face (cheaper than a division on GB300's float64
-        // pipe); exact scaling, so bit-identical to 2/(rho_L + rho_R)/h^2 when h is
-        // a power of two, within 2 ulp otherwise
-        const double gxm = face_minus(i, g.nx, g.bcx) ? c2x * __drcp_rn(rn + rho_new[nbr_x(idx, i, g).im]) : 0.0;
-        const double gym = face_minus(j, g.ny, g.bcy) ? c2y * __drcp_rn(rn + rho_new[nbr_y(idx, j, g).im]) : 0.0;
-        const double gzm = face_minus(k, g.nz, g.bcz) ? c2z * __drcp_rn(rn + rho_new[nbr_z(idx, k, g).im]) : 0.0;
+        // mean), evaluated as (2/h^2) * RN(1/(rho_L + rho_R)): exact scaling, so
+        // bit-identical to 2/(rho_L + rho_R)/h^2 when h is a power of two, within
+        // 2 ulp otherwise.  The four reciprocals, the tests and the conversions
+        // run on the integer pipe (lm_intfp.cuh), which leaves the float64 pipe
+        // five sums and products a cell and one more per axis whose 2/h^2 is no
+        // power of two: 256^3 1062 -> 439 us
+        const double gxm =
+            face_minus(i, g.nx, g.bcx) ? mul_pow2(ircp(rn + rho_new[nbr_x(idx, i, g).im]), c2x, a.kx) : 0.0;
+        const double gym =
+            face_minus(j, g.ny, g.bcy) ? mul_pow2(ircp(rn + rho_new[nbr_y(idx, j, g).im]), c2y, a.ky) : 0.0;
+        const double gzm =
+            face_minus(k, g.nz, g.bcz) ? mul_pow2(ircp(rn + rho_new[nbr_z(idx, k, g).im]), c2z, a.kz) : 0.0;
         out.ct[idx] = c;
         out.gx[idx] = gxm;
         out.gy[idx] = gym;
         out.gz[idx] = gzm;
-        const float c32 = (float)c;
+        const float c32 = to_f32(c);
         bad32 = bad32 || !(c32 > 0.f) || isinf(c32);
         out.ct32[idx] = c32;
-        out.rho32[idx] = (float)rn;
+        out.rho32[idx] = to_f32(rn);
     }
     // the block's range and float32 flag: one atomic per warp
     for (int o = 16; o > 0; o >>= 1) {
