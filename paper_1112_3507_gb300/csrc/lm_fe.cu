@@ -194,6 +194,82 @@ __device__ __forceinline__ T bx_point(int idx, const FeOp<T>& op, LD ld, T& xc) 
     return op.vc[idx] * xc + st;
 }
 
+// The same in 3D and float64 with the stiffness sums in integers (lm_intfp.cuh),
+// one a class, or one for the three classes of edges where their c is the same
+// (cubic elements).  The float64 form takes 82 issue slots of its pipe a point, at
+// 18.5 cycles an SM; this takes about 750 integer instructions: the residual of
+// 256^3 points 2771 -> 947 us.
+template <bool FACES>
+__device__ __forceinline__ double bx3_fix(int idx, const FeOp<double>& op, const double* x) {
+    constexpr int XB = 5, GB = 3;
+    const FeGeo& g = op.g;
+    int i, j, k;
+    coords(idx, g, i, j, k);
+    const int sz = g.nx * g.ny;
+    const int cx[3] = {wrap_m(i, g.nx), i, wrap_p(i, g.nx)};
+    const int ry[3] = {wrap_m(j, g.ny) * g.nx, j * g.nx, wrap_p(j, g.ny) * g.nx};
+    const int pz[3] = {wrap_m(k, g.nz) * sz, k * sz, wrap_p(k, g.nz) * sz};
+    uint64_t X[27], E[2][2][2];
+    lm::ExpRange rx, re;
+#pragma unroll
+    for (int o = 0; o < 27; ++o)
+        if (o == 13 || FACES || (o % 3 != 1) + (o / 3 % 3 != 1) + (o / 9 != 1) > 1) {
+            X[o] = (uint64_t)__double_as_longlong(x[pz[o / 9] + ry[o / 3 % 3] + cx[o % 3]]);
+            rx.add((uint32_t)(X[o] >> 32) & 0x7fffffffu);
+        }
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        uint64_t& e = E[d >> 2][d >> 1 & 1][d & 1];
+        e = (uint64_t)__double_as_longlong(op.ke[pz[1 - (d >> 2)] + ry[1 - (d >> 1 & 1)] + cx[1 - (d & 1)]]);
+        re.add((uint32_t)(e >> 32));
+    }
+    if (!lm::fix_ok(rx, XB, re, GB)) {
+        double xc;
+        return bx_point(idx, op, [&](int j) { return x[j]; }, xc);
+    }
+    const int ex = rx.top(), ee = re.top(), e0 = lm::fix_scale<XB, GB>(ex, ee);
+    const lm::Limbs c0 = lm::fix<XB>(X[13], ex);
+    lm::Limbs L[2][2][2];
+#pragma unroll
+    for (int d = 0; d < 8; ++d) L[d >> 2][d >> 1 & 1][d & 1] = lm::fix_abs<GB>(E[d >> 2][d >> 1 & 1][d & 1], ee);
+    auto sum = [&](int cls) {
+        lm::FixSum s;
+#pragma unroll
+        for (int o = 0; o < 27; ++o) {
+            const int ox = o % 3 - 1, oy = o / 3 % 3 - 1, oz = o / 9 - 1;
+            if (((ox != 0) | ((oy != 0) << 1) | ((oz != 0) << 2)) != cls) continue;
+            lm::Limbs K{0, 0};
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                const int dx = d & 1, dy = d >> 1 & 1, dz = d >> 2;
+                if ((ox == 1 && dx) || (ox == -1 && !dx) || (oy == 1 && dy) || (oy == -1 && !dy) || (oz == 1 && dz) ||
+                    (oz == -1 && !dz))
+                    continue;
+                K.h += L[dz][dy][dx].h;
+                K.l += L[dz][dy][dx].l;
+            }
+            // (B x)_i holds x_{i+o} - x_i: the sign goes to the class's factor
+            s.mac(lm::fix_diff<XB>(c0, X[o], ex), K);
+        }
+        return s.total();
+    };
+    auto rnd = [&](__int128 t) { return __longlong_as_double((long long)lm::fix_round(t, e0)); };
+    double y = op.vc[idx] * __longlong_as_double((long long)X[13]);
+    if (FACES) {
+#pragma unroll
+        for (int cls = 1; cls < 7; ++cls) y -= op.c[cls] * rnd(sum(cls));
+    } else {
+        if (op.c[3] == op.c[5] && op.c[3] == op.c[6]) {
+            y -= op.c[3] * rnd(sum(3) + sum(5) + sum(6));
+        } else {
+            y -= op.c[3] * rnd(sum(3));
+            y -= op.c[5] * rnd(sum(5));
+            y -= op.c[6] * rnd(sum(6));
+        }
+    }
+    return y - op.c[7] * rnd(sum(7));
+}
+
 // ---- set-up -----------------------------------------------------------------
 
 struct FeFlags {
@@ -205,7 +281,7 @@ using lm::pos_finite;
 // 0, or 2^-125 < |v| < 2^126, by the bits
 __device__ __forceinline__ bool normal32(double v) {
     const uint64_t m = (uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
-    return m == 0 || (m > (898ull << 52) && m < (1149ull << 52));
+    return m << 1 == 0 || (m > (898ull << 52) && m < (1149ull << 52));
 }
 
 // kappa_e of the element with lowest corner idx (0 past a wall) and V c~.
@@ -341,22 +417,28 @@ __global__ void __launch_bounds__(NT) k_fe_resid64(FeOp<double> op, const double
 
 // Refinement residual: r = f - B x, r32 = r * rscale (a power of two);
 // the last block sets st->rel = ||r|| / ||f|| (and st->fnorm when SET_FNORM).
-template <bool SET_FNORM>
+// D3: 0 in 2D; in 3D 1, or 2 where the faces have weights; -1 for x = 0 (which it
+// sets), r = f, without the stencil's registers.
+template <bool SET_FNORM, int D3>
 __global__ void __launch_bounds__(NT) k_fe_ir_res64(FeOp<double> op, const double* __restrict__ f, double* x,
-                                                    float* __restrict__ r32, int zero_x, double rscale, int kscale,
-                                                    Red red, SolveState* st) {
+                                                    float* __restrict__ r32, double rscale, int kscale, Red red,
+                                                     SolveState* st) {
     __shared__ double sm[64];
     double acc[2] = {0.0, 0.0};
     auto ld = [&](int j) { return x[j]; };
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < op.g.N; idx += gridDim.x * blockDim.x) {
         const double fi = f[idx];
         double xc;
-        const double ri = zero_x ? fi : fi - bx_point(idx, op, ld, xc);
-        if (zero_x) x[idx] = 0.0;
+        double ri = fi;
+        if (D3 < 0)
+            x[idx] = 0.0;
+        else
+            ri -= D3 == 0 ? bx_point(idx, op, ld, xc) : bx3_fix<D3 == 2>(idx, op, x);
         r32[idx] = lm::to_f32(lm::mul_pow2(ri, rscale, kscale));
         acc[0] += ri * ri;
-        if (SET_FNORM) acc[1] += fi * fi;             // ||f|| is kept from the first residual
+        if (SET_FNORM && D3 >= 0) acc[1] += fi * fi;  // ||f|| is kept from the first residual
     }
+    if (D3 < 0) acc[1] = acc[0];
     const int sl[2] = {SLOT_RR, SLOT_FF};
     if (lm::grid_reduce<2>(acc, red, sl, sm) && threadIdx.x == 0) {
         if (SET_FNORM) st->fnorm = sqrt(red.scal[SLOT_FF]);
@@ -685,12 +767,16 @@ void launch_fe32(const lm_fe* fe, cudaStream_t s, const FeIO32& io, int dots = 0
 void launch_fe_ir_res(const lm_fe* fe, cudaStream_t s, int zero_x, int set_fnorm, double rscale) {
     lm::count_launches(1);
     const FeOp<double> op = fe_op<double>(fe);
-    if (set_fnorm)
-        k_fe_ir_res64<true><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, lm::pow2_of(rscale),
-                                                      fe_red(fe), fe->st);
-    else
-        k_fe_ir_res64<false><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, zero_x, rscale, lm::pow2_of(rscale),
-                                                      fe_red(fe), fe->st);
+#define LM_FEIR(F, D)                                                                                        \
+    k_fe_ir_res64<F, D><<<fe->G, NT, 0, s>>>(op, fe->f, fe->x, fe->r32, rscale, lm::pow2_of(rscale), \
+                                             fe_red(fe), fe->st)
+    const int d3 = zero_x ? -1 : fe->geo.dim == 3 ? 1 + (fe->faces != 0) : 0;
+    if (set_fnorm) {
+        if (d3 < 0) LM_FEIR(true, -1); else if (d3 == 0) LM_FEIR(true, 0); else if (d3 == 1) LM_FEIR(true, 1); else LM_FEIR(true, 2);
+    } else {
+        if (d3 < 0) LM_FEIR(false, -1); else if (d3 == 0) LM_FEIR(false, 0); else if (d3 == 1) LM_FEIR(false, 1); else LM_FEIR(false, 2);
+    }
+#undef LM_FEIR
 }
 
 lm::PcgArgs fe_pcg_args(lm_fe* fe, int max_iter) {

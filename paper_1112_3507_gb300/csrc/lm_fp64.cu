@@ -503,23 +503,25 @@ __global__ void __launch_bounds__(NT) k_finish_rel(double* part, int G, SolveSta
 // launcher asks for it when the residual's expected size is well inside
 // float32 range; it saves a float64 multiply a cell on GB300's slow float64
 // pipe); 2 scaled in float64 before rounding.
-template <bool FNORM, int SC>
+// ZERO: x = 0 (which it sets), so r = f: a kernel of its own, since the stencil's
+// registers would leave this one, bound by memory, too few warps (256^3: 111 -> 82 us).
+template <bool FNORM, int SC, bool ZERO>
 __global__ void __launch_bounds__(NT) k_ir_residual(Geo g, Op64 op, const double* __restrict__ f,
                                                     double* __restrict__ x, float* __restrict__ r32,
-                                                    double* __restrict__ part, int zero_x, double rscale) {
+                                                    double* __restrict__ part, double rscale) {
     __shared__ double sm[64];
     double acc[2] = {0.0, 0.0};
     const float rs32 = (float)rscale;
     const int stride = gridDim.x * blockDim.x;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx += stride) {
         const double fi = f[idx];
-        const double ri = zero_x ? fi : fi - apply64_at(idx, g, op, x);
+        const double ri = ZERO ? fi : fi - apply64_fix(idx, g, op, x);
+        if (ZERO) x[idx] = 0.0;
         r32[idx] = SC == 2 ? (float)(ri * rscale) : (SC == 1 ? to_f32(ri) * rs32 : to_f32(ri));
         acc[0] += ri * ri;
-        if (FNORM) acc[1] += fi * fi;
+        if (FNORM && !ZERO) acc[1] += fi * fi;
     }
-    if (zero_x)
-        for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx += stride) x[idx] = 0.0;
+    if (ZERO) acc[1] = acc[0];
     block_sum<2>(acc, sm);
     if (threadIdx.x == 0) {
         part[1 * MAX_PARTIALS + blockIdx.x] = acc[0];
@@ -761,12 +763,17 @@ void launch_ir_residual(const Geo& g, int G, cudaStream_t s, const Op64& op, con
     // rscale near 1/rms(r): the residual's size is about 1/rscale, a normal
     // float32 (with room for small entries) when rscale is within 2^+-90
     const int sc = rscale == 1.0 ? 0 : (rscale >= 0x1p-90 && rscale <= 0x1p90 ? 1 : 2);
-#define LM_IRR(F, SC) k_ir_residual<F, SC><<<G, NT, 0, s>>>(g, op, f, x, r32, part, zero_x, rscale)
-    if (set_fnorm) {
-        if (sc == 0) LM_IRR(true, 0); else if (sc == 1) LM_IRR(true, 1); else LM_IRR(true, 2);
+#define LM_IRR(F, SC, Z) k_ir_residual<F, SC, Z><<<G, NT, 0, s>>>(g, op, f, x, r32, part, rscale)
+#define LM_IRR_SC(F, Z) \
+    do {                \
+        if (sc == 0) LM_IRR(F, 0, Z); else if (sc == 1) LM_IRR(F, 1, Z); else LM_IRR(F, 2, Z); \
+    } while (0)
+    if (zero_x) {
+        if (set_fnorm) LM_IRR_SC(true, true); else LM_IRR_SC(false, true);
     } else {
-        if (sc == 0) LM_IRR(false, 0); else if (sc == 1) LM_IRR(false, 1); else LM_IRR(false, 2);
+        if (set_fnorm) LM_IRR_SC(true, false); else LM_IRR_SC(false, false);
     }
+#undef LM_IRR_SC
 #undef LM_IRR
     count_launches(1);
     k_finish_rel<<<1, NT, 0, s>>>(part, G, st, set_fnorm, hist_entry);

@@ -29,7 +29,8 @@
 // About 65 integer instructions, against seven (reciprocal) and eleven
 // (quotient) issue slots of the float64 pipe at 18.5 cycles an SM each.
 //
-// Sign, finiteness and order of float64 values are those of their bits; a
+// Sign, finiteness and order of float64 values are those of their bits (a zero is
+// tested by a shift: the compiler makes a float64 comparison of a masked test); a
 // conversion between normal float32 and float64 values shifts the mantissa.
 #pragma once
 
@@ -117,7 +118,7 @@ __device__ __forceinline__ float to_f32(double v) {
         const uint32_t r = (uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29) - (896u << 23);
         return __uint_as_float(r | (uint32_t)(u >> 32 & 0x80000000u));
     }
-    if (!m) return __uint_as_float((uint32_t)(u >> 32));
+    if (!(u << 1)) return __uint_as_float((uint32_t)(u >> 32));
     return (float)v;
 }
 // (double)v
@@ -141,6 +142,128 @@ __device__ __forceinline__ double mul_pow2(double v, double factor, int k) {
     return v * factor;
 }
 #endif
+
+// a b > 0 ? (|a| < |b| ? a : b) : 0 on the bits of a and b, the product rounded to
+// float64 as the comparison with it would have it (so zero below 2^-1075).  No
+// float64 instruction even in the rare case, which a compiler would run for all.
+LM_HD uint64_t minmod_bits(uint64_t a, uint64_t b) {
+    const uint64_t M = 0x7fffffffffffffffull, ma = a & M, mb = b & M;
+    if (!(a << 1) || !(b << 1) || (int64_t)(a ^ b) < 0) return 0;
+    if ((uint32_t)(ma >> 32) - 0x20000000u >= 0x5ff00000u || (uint32_t)(mb >> 32) - 0x20000000u >= 0x5ff00000u) {
+        const uint64_t inf = 0x7ffull << 52;
+        if (ma > inf || mb > inf) return 0;                    // NaN
+        if (ma < inf && mb < inf) {
+            const int ea = (int)(ma >> 52), eb = (int)(mb >> 52);
+            const uint64_t A = (ma & ((1ull << 52) - 1)) | (ea ? 1ull << 52 : 0),
+                           B = (mb & ((1ull << 52) - 1)) | (eb ? 1ull << 52 : 0);
+            const int t = 1075 - (ea ? ea : 1) - (eb ? eb : 1);   // a b = A B 2^(-1075 - t)
+            if (t > 106) return 0;
+            if (t >= 0 && (unsigned __int128)A * B <= (unsigned __int128)1 << t) return 0;
+        }
+    }
+    return ma < mb ? a : b;
+}
+
+// ---- exact stencil sums ---------------------------------------------------------
+//
+// sum_o g_o (x_c - x_o) over neighbours of a cell, in integers.  The x become
+// integers at one scale, of 53 + XB bits where the largest x has its leading one,
+// and the weights likewise with GB; both as limbs h 2^29 + l, the x with their sign
+// on both limbs, so that differences and sums of weights need no carry.  Products
+// accumulate exactly in three 64-bit sums, four widening multiply-adds a term, and
+// the total is rounded once to float64.
+//
+// Precision.  Where the nonzero x lie within 2^XB of each other and the weights
+// within 2^GB the sum is exact before its one rounding; float64 rounds every
+// difference, product and partial sum.  An x further down is cut off at 2^-(52 + XB)
+// of the largest, E: a term is off by less than 2^-(51 + XB) g E.  Then some
+// difference is at least E / 2 in magnitude, and the float64 form rounds it, its
+// product and the partial sums after that by up to 2^-53 of them each -- with XB = 5
+// 8 times the cut for as large a weight.  So x of any spread are taken where the
+// weights lie within a factor of four; all else takes the float64 form.
+//
+// Room: |xl|, |xh| < 2^29 with XB <= 5, so differences < 2^30; gl < 2^29 and
+// gh < 2^(24 + GB) <= 2^28.  Six single weights, or FE's sums of two (four terms) and
+// four (two terms) with GB = 3, keep each sum below 2^62.5.
+
+// range of the nonzero magnitudes, by their high words
+struct ExpRange {
+    uint32_t hi = 0, lo = 0xffffffffu;      // largest; smallest nonzero, less one
+    LM_HD void add(uint32_t h) {            // h: high word without its sign
+        hi = h > hi ? h : hi;
+        lo = h - 1u < lo ? h - 1u : lo;
+    }
+    LM_HD int top() const { return (int)(hi >> 20); }
+    LM_HD int spread() const { return (int)(hi >> 20) - (int)((lo + 1u) >> 20); }
+};
+// both ranges in reach, and the sum's exponent in the normal range however far
+// its terms cancel (zeros are below every scale: 2^200 over the smallest normal)
+LM_HD bool fix_ok(const ExpRange& x, int xb, const ExpRange& g, int gb) {
+    const int ex = x.top(), eg = g.top(), sg = g.spread();
+    return ex >= 200 && ex < 2047 && eg >= 200 && eg < 2047 && sg <= gb && (x.spread() <= xb || sg <= 1) &&
+           (unsigned)(ex + eg - 1023 - 150) < 1880u;
+}
+struct Limbs {
+    int32_t h, l;
+};
+// |v| of the value's bits at scale 2^(52 + B) over exponent `top`
+template <int B>
+LM_HD Limbs fix_abs(uint64_t u, int top) {
+    const int sh = top - ((int)(u >> 52) & 0x7ff);
+    const uint64_t m = (((u & ((1ull << 52) - 1)) | (1ull << 52)) << B) >> (sh > 63 ? 63 : sh);
+    return {(int32_t)(uint32_t)(m >> 29), (int32_t)((uint32_t)m & 0x1fffffffu)};
+}
+template <int B>
+LM_HD Limbs fix(uint64_t u, int top) {
+    const Limbs a = fix_abs<B>(u, top);
+    const int32_t s = (int32_t)((int64_t)u >> 63) | 1;
+    return {a.h * s, a.l * s};
+}
+// c - v
+template <int B>
+LM_HD Limbs fix_diff(Limbs c, uint64_t u, int top) {
+    const Limbs a = fix_abs<B>(u, top);
+    const int32_t s = ~(int32_t)((int64_t)u >> 63) | 1;
+    return {c.h + a.h * s, c.l + a.l * s};
+}
+struct FixSum {
+    int64_t a0 = 0, a1 = 0, a2 = 0;         // weights 1, 2^29, 2^58
+    LM_HD void mac(Limbs d, Limbs g) {
+        a0 += (int64_t)d.l * g.l;
+        a1 += (int64_t)d.l * g.h;
+        a1 += (int64_t)d.h * g.l;
+        a2 += (int64_t)d.h * g.h;
+    }
+    LM_HD __int128 total() const { return ((__int128)a2 << 58) + ((__int128)a1 << 29) + a0; }
+};
+// t rounded to float64, as bits; e: the exponent field of 2^0 at t's scale
+LM_HD uint64_t fix_round(__int128 t, int e) {
+    const uint64_t s = (uint64_t)((int64_t)(t >> 64) >> 63);
+    uint64_t lo = (uint64_t)t ^ s, hi = (uint64_t)(t >> 64) ^ s;
+    lo -= s;
+    hi += s & (uint64_t)(lo == 0);
+    if (!hi) {                               // |t| < 2^64
+        if (!lo) return 0;
+        hi = lo;
+        lo = 0;
+        e -= 64;
+    }
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)hi);
+#else
+    const int z = __builtin_clzll(hi);
+#endif
+    uint64_t m = hi << z | (lo >> 1) >> (63 - z);
+    m |= (uint64_t)(lo << z != 0);
+    m = (m >> 11) + (((m & 0x7ff) + 0x3ff + ((m >> 11) & 1)) >> 11);
+    return (m + ((uint64_t)(e + 126 - z) << 52)) | (s & (1ull << 63));
+}
+// the exponent field of 2^0 at the scale of a sum of x (top ex) times g (top eg)
+template <int XB, int GB>
+LM_HD int fix_scale(int ex, int eg) {
+    return ex + eg - 1023 - 104 - XB - GB;
+}
+
 // the exponent k of a factor 2^k, else POW2_NONE (host)
 inline int pow2_of(double f) {
     int e = 0;

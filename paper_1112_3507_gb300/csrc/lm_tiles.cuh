@@ -31,6 +31,45 @@ __device__ __forceinline__ double apply64_at(int idx, const Geo& g, const Op64& 
     return y;
 }
 
+// The same with the x and y faces' terms summed exactly in integers (lm_intfp.cuh)
+// and the z faces' on the float64 pipe: that pipe takes 18.5 cycles an SM for each
+// of its instructions, the integer form of two faces about as long as four of them,
+// so the two run side by side.  It wins where the float64 pipe is the bound, in
+// grids of many cells an SM (256^3 residual: 500 us in float64 alone, 400 with all
+// six faces in integers, 333 so); where latency is it makes no difference.
+__device__ __forceinline__ double apply64_fix(int idx, const Geo& g, const Op64& op, const double* __restrict__ x) {
+    constexpr int XB = 5, GB = 4;
+    int i, j, k;
+    cell_coords(idx, g, i, j, k);
+    const bool y = g.ny > 1;
+    const Nbr nx = nbr_x(idx, i, g), nz = nbr_z(idx, k, g), ny = y ? nbr_y(idx, j, g) : nx;
+    const double xc = x[idx];
+    const uint64_t uc = (uint64_t)__double_as_longlong(xc);
+    uint64_t X[4], W[4];
+    auto ld = [](const double* p, int q) { return (uint64_t)__double_as_longlong(p[q]); };
+    X[0] = ld(x, nx.im), X[1] = ld(x, nx.ip), W[0] = ld(op.gx, idx), W[1] = ld(op.gx, nx.ip);
+    if (y) X[2] = ld(x, ny.im), X[3] = ld(x, ny.ip), W[2] = ld(op.gy, idx), W[3] = ld(op.gy, ny.ip);
+    const double c = op.ct[idx], zm = x[nz.im], zp = x[nz.ip], wm = op.gz[idx], wp = op.gz[nz.ip];
+    ExpRange rx, rw;
+    rx.add((uint32_t)(uc >> 32) & 0x7fffffffu);
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+        if (o < 2 || y) rx.add((uint32_t)(X[o] >> 32) & 0x7fffffffu), rw.add((uint32_t)(W[o] >> 32));
+    if (fix_ok(rx, XB, rw, GB)) {
+        const int ex = rx.top(), ew = rw.top();
+        const Limbs c0 = fix<XB>(uc, ex);
+        FixSum s;
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+            if (o < 2 || y) s.mac(fix_diff<XB>(c0, X[o], ex), fix_abs<GB>(W[o], ew));
+        double v = fma(c, xc, __longlong_as_double((long long)fix_round(s.total(), fix_scale<XB, GB>(ex, ew))));
+        v += wm * (xc - zm);
+        v += wp * (xc - zp);
+        return v;
+    }
+    return apply64_at(idx, g, op, x);
+}
+
 // Coefficient assembly (step (v); Eqs. cpoiss, kappapoiss) of the cells
 // start, start + stride, ... of one grid, with the range of rho^{n+1} and
 // the failure flags reduced per warp into a.fl (every lane of a warp must

@@ -1,6 +1,6 @@
-"""The integer-pipe float64 quotient: its arithmetic compiled for the host and
-compared with the hardware division, and the device's own through the entry
-points that use it."""
+"""Float64 quotients and stencil sums on the integer pipe: their arithmetic compiled
+for the host and compared with the hardware division and with integers, and the
+device's own through the entry points that use it."""
 import os
 import shutil
 import subprocess
@@ -11,6 +11,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1112_3507_gb300", "csrc")
 
 PROGRAM = r"""
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <random>
@@ -50,13 +51,55 @@ int main() {
         const double b = value((g() & M) | ((uint64_t)(600 + g() % 800) << 52));
         bad += quotient(a, b, (int)(i % 5) - 2) != a / b;
     }
+    // minmod over all magnitudes, signs, zeros, subnormals, infinities and NaN
+    for (long i = 0; i < 1000000; ++i) {
+        auto any = [&] {
+            const int e = i % 3 == 0 ? g() % 2048 : i % 3 == 1 ? 480 + g() % 64 : (g() & 1 ? 0 : 1020 + g() % 60);
+            const uint64_t m = g() % 5 == 0 ? 0 : g() % 5 == 0 ? 1 : g() & M;
+            return (uint64_t)e << 52 | m | (g() & 1) << 63;
+        };
+        const uint64_t u = any(), v = g() % 16 == 0 ? u : any();
+        const double a = value(u), b = value(v);
+        bad += lm::minmod_bits(u, v) != bits(a * b > 0.0 ? (fabs(a) < fabs(b) ? a : b) : 0.0);
+    }
+    // sums of products of differences, against integers: mantissas A, B of 53 bits,
+    // x = +-A 2^p with p < 6, w = B 2^q with q < 5, or zero
+    for (long i = 0; i < 300000; ++i) {
+        const int mode = i % 4, p0 = (int)(g() % 1200) - 600, q0 = (int)(g() % 600) - 300;
+        int64_t X[7], W[6];
+        uint64_t xu[7], wu[6];
+        lm::ExpRange rx, rw;
+        auto mant = [&] { return (int64_t)(mode == 0 ? M - (g() & 3) : mode == 1 ? g() & 3 : g() & M) | (1ll << 52); };
+        for (int o = 0; o < 7; ++o) {
+            const int64_t p = mode == 3 ? 5 : g() % 6, a = g() % 11 ? mant() : 0;
+            X[o] = g() & 1 && mode != 3 ? -(a << p) : a << p;
+            xu[o] = a ? ((uint64_t)(p0 + p + 1075) << 52 | (a & M)) | (X[o] < 0 ? 1ull << 63 : 0) : 0;
+            rx.add((uint32_t)(xu[o] >> 32) & 0x7fffffffu);
+        }
+        for (int o = 0; o < 6; ++o) {
+            const int64_t q = g() % 5, b = g() % 7 ? mant() : 0;
+            W[o] = b << q;
+            wu[o] = b ? (uint64_t)(q0 + q + 1075) << 52 | (b & M) : 0;
+            rw.add((uint32_t)(wu[o] >> 32));
+        }
+        if (!lm::fix_ok(rx, 5, rw, 4)) continue;
+        const lm::Limbs c = lm::fix<5>(xu[6], rx.top());
+        lm::FixSum s;
+        __int128 S = 0;
+        for (int o = 0; o < 6; ++o) {
+            s.mac(lm::fix_diff<5>(c, xu[o], rx.top()), lm::fix_abs<4>(wu[o], rw.top()));
+            S += (__int128)(X[6] - X[o]) * W[o];
+        }
+        const uint64_t e = lm::fix_scale<5, 4>(rx.top(), rw.top());
+        bad += value(lm::fix_round(s.total(), (int)e)) != ldexp((double)S, p0 + q0);
+    }
     printf("%ld\n", bad);
     return bad != 0;
 }
 """
 
 
-def test_quotient_on_the_host(tmp_path):
+def test_arithmetic_on_the_host(tmp_path):
     gxx = shutil.which("g++")
     if not gxx:
         pytest.skip("no g++")
@@ -139,3 +182,59 @@ def test_assembly_bits(lm, h):
     assert np.array_equal(c32.cpu().numpy(), ct.astype(np.float32))
     assert np.array_equal(r32.cpu().numpy() * np.float32(scale.value), rn.astype(np.float32))
     g.close()
+
+
+def _field(kind, N, rng):
+    if kind == "near one":
+        return 1.0 + 1e-6 * rng.standard_normal(N)
+    if kind == "both signs":
+        return rng.standard_normal(N) * 1e-30
+    x = rng.standard_normal(N) * 2.0 ** rng.integers(-40, 40, N)      # wide
+    x[rng.random(N) < 0.2] = 0.0
+    return x
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,h", [((40, 1, 37), (1 / 32, 1.0, 1 / 32)), ((34, 10, 12), (0.1, 0.2, 0.15)), ((64, 24, 32), (1 / 64,) * 3)])
+@pytest.mark.parametrize("kind", ["near one", "both signs", "wide"])
+@pytest.mark.parametrize("spread", [0.05, 3.0])
+def test_refinement_residuals(lm, n, h, kind, spread):
+    """f - A x of the solvers' refinement where f is A x from the float64 apply: only
+    the rounding of the row's terms is left, (terms + 2) half units of their sum each."""
+    import torch
+    rng = np.random.default_rng(n[0])
+    N = n[0] * n[1] * n[2]
+    shape = (n[2], n[1], n[0])
+    rho = np.exp(rng.uniform(-spread, spread, N))
+    ct = np.exp(rng.uniform(-1.0, 1.0, N))
+    x = _field(kind, N, rng)
+    bc = (0, 0, 1)
+    d = lambda a: torch.as_tensor(a, device="cuda")
+    ndim = 2 if n[1] == 1 else 3
+    with lm.Grid(n, h, bc) as g:
+        g.set_coefficients_raw(ct, rho)
+        f = d(np.empty(N))
+        g.apply(d(x), f)
+        g.set_rhs(f)
+        g.set_initial_guess(d(x))
+        rel = g.solve(rtol=1.0, use_x0=1)["rel_residual"]
+        c, *gs = (t.cpu().numpy().reshape(shape) for t in g.coefficients())
+    xs = x.reshape(shape)
+    mag = np.abs(c * xs)
+    for a, gm in enumerate(gs):
+        t = gm * np.abs(xs - np.roll(xs, 1, 2 - a))
+        mag += t + np.roll(t, -1, 2 - a)
+    tol = lambda mag, terms, f: 2 * (terms + 2) * 2.0 ** -53 * np.linalg.norm(mag) / np.linalg.norm(f)
+    assert rel <= tol(mag, 7, f.cpu().numpy())
+    from oracle import fem as F
+    op = F.FEOperator(ct.reshape(shape), rho.reshape(shape), h, bc)
+    with lm.FEGrid(n, h, bc) as fe:
+        fe.set_coefficients(ct, rho)
+        fe.apply(d(x), f)
+        rel = fe.solve(f, d(x), rtol=1.0, use_x0=1)["rel_residual"]
+    mag = np.abs(op.volume * op.ct * xs)
+    xc = [op._corner(xs, c) for c in op.corners]
+    for p in range(len(op.corners)):
+        for q in range(len(op.corners)):
+            mag += op._back(op.kappa_e * abs(op.kref[p, q]) * np.abs(xc[q] - xc[p]), op.corners[p])
+    assert rel <= tol(mag, 27, f.cpu().numpy())
