@@ -11,10 +11,17 @@
 //                  c_s^2 = gamma P / rho for the next step's c~.
 //
 // A wall face carries no flux and a cell next to a wall has zero slope (its
-// outer neighbour does not exist); periodic axes wrap.  One thread per
-// cell computes both faces of each axis it needs (the face fluxes are
-// recomputed by the two cells that share them), so the kernel needs no
-// synchronisation; the float64 pipe bounds it on GB300.
+// outer neighbour does not exist); periodic axes wrap.
+//
+// The float64 pipe bounds it on GB300 (one warp instruction per 18.5 cycles an
+// SM), so every difference, slope and face flux is formed once, in one pass an
+// axis, and every comparison and quotient runs on the integer pipe
+// (lm_intfp.cuh): five float64 instructions a quantity, cell and axis where one
+// thread a cell, forming both faces of every axis, took 22.  Along y and z a
+// thread marches up a chunk of a column and keeps the last face in registers;
+// along x the lanes of a warp hold successive cells and pass differences, slopes
+// and fluxes by shuffles.  The passes after the first add to the outputs.
+// Five quantities on 96^3 791 -> 234 us, on 256^2 52 -> 25 us.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -28,12 +35,13 @@ namespace {
 constexpr int MAXQ = 6;       // rho, rho u (3), e, rho c
 
 struct AdvGeo {
-    int n[3];
-    int N;
-    int wall[3];
-    double rh[3];             // 1 / h
-    int stride[3];
-    int nq;                   // 5, or 6 with rho c
+    int n;                    // cells along the pass's axis
+    int stride;               // between them
+    int wall;
+    int rows;                 // columns of the axis: N / n
+    int inner, outer;         // column q starts at (q / inner) outer + q % inner
+    int L;                    // cells a thread (y and z)
+    double k;                 // dt / h
 };
 
 struct AdvIO {
@@ -42,68 +50,160 @@ struct AdvIO {
 };
 
 __device__ __forceinline__ double minmod(double a, double b) {
-    return a * b > 0.0 ? (fabs(a) < fabs(b) ? a : b) : 0.0;
+    return __longlong_as_double(
+        (long long)lm::minmod_bits((uint64_t)__double_as_longlong(a), (uint64_t)__double_as_longlong(b)));
 }
 
-// index of the cell at offset t (|t| <= 2) along an axis from position c:
-// wrapped on a periodic axis, clamped on a wall axis (clamped values are
-// never used: wall cells have zero slope and the wall face no flux)
-__device__ __forceinline__ int along(int idx, int c, int t, int n, int stride, int wall) {
-    int d = c + t;
-    if (wall) {
-        d = d < 0 ? 0 : (d >= n ? n - 1 : d);
-    } else {
-        d = d < 0 ? d + n : (d >= n ? d - n : d);
-    }
-    return idx + (d - c) * stride;
+// offset along an axis of the cell at position d in [-2, n + 1]: wrapped on a
+// periodic axis, clamped on a wall axis (clamped values are never used: wall
+// cells have zero slope and the wall face no flux)
+__device__ __forceinline__ int along(int d, int n, int wall) {
+    if (d < 0) return wall ? 0 : d + n;
+    if (d >= n) return wall ? n - 1 : d - n;
+    return d;
 }
 
-__global__ void __launch_bounds__(lm::NT) k_advect(AdvGeo G, AdvIO io, double dt) {
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < G.N; idx += gridDim.x * blockDim.x) {
-        int c[3];
-        c[0] = idx % G.n[0];
-        const int t = idx / G.n[0];
-        c[1] = t % G.n[1];
-        c[2] = t / G.n[1];
-        double acc[MAXQ];
-        for (int q = 0; q < G.nq; ++q) acc[q] = io.q[q][idx];
-        for (int a = 0; a < 3; ++a) {
-            const int n = G.n[a];
-            if (n == 1) continue;
-            const int s = G.stride[a], w = G.wall[a];
-            int id[5];
+// (dt / h) u of the minus face of the cell at position c (Eq. step1), cells m and c
+__device__ __forceinline__ double face_w(const AdvGeo& G, int c, double rm, double rc, double mm, double mc) {
+    return G.wall && (c == 0 || c == G.n) ? 0.0 : G.k * lm::idiv(mm + mc, rm + rc);
+}
+// (dt / h) times a quantity's flux through it: the upwind side's value at the face
+__device__ __forceinline__ double face_flux(double w, double xm, double sm, double xc, double sc) {
+    const bool up = __double_as_longlong(w) > 0;
+    return fma(up ? 0.5 : -0.5, up ? sm : sc, up ? xm : xc) * w;
+}
+__device__ __forceinline__ bool flat_at(const AdvGeo& G, int c) { return G.wall && (c <= 0 || c >= G.n - 1); }
+
+// The pass along x, the first where nx > 1.  A row's items are its positions -1 ..
+// n + 1; a warp takes 32 successive items of all rows and writes the 29 whose
+// difference, slopes and fluxes its lanes hold.
+template <int NQ>
+__global__ void __launch_bounds__(lm::NT) k_advect_x(AdvGeo G, AdvIO io) {
+    constexpr int OUT = 29;
+    const int lane = threadIdx.x & 31;
+    const uint64_t m = (uint64_t)G.n + 3, items = (uint64_t)G.rows * m;
+    const uint64_t warps = (items + OUT - 1) / OUT, step = (uint64_t)gridDim.x * (lm::NT / 32);
+    const bool small = items + 64 < (1ull << 32);
+    for (uint64_t w0 = (uint64_t)blockIdx.x * (lm::NT / 32) + threadIdx.x / 32; w0 < warps; w0 += step) {
+        uint64_t it = w0 * OUT + lane;
+        const bool in = it < items;
+        if (!in) it = items - 1;
+        const int row = small ? (int)((uint32_t)it / (uint32_t)m) : (int)(it / m);
+        const int c = (int)(it - (uint64_t)row * m) - 1;
+        const int base = row * G.n, ic = base + along(c, G.n, G.wall), im = base + along(c - 1, G.n, G.wall);
+        double xc[NQ], xm[NQ];
 #pragma unroll
-            for (int o = 0; o < 5; ++o) id[o] = along(idx, c[a], o - 2, n, s, w);
-            // slope use: a wall axis' end cells have zero slope
-            bool flat[5];
+        for (int q = 0; q < NQ; ++q) xc[q] = io.q[q][ic], xm[q] = io.q[q][im];
+        const double w = face_w(G, c, xm[0], xc[0], xm[1], xc[1]);
+        const bool flat = flat_at(G, c), put = in && lane >= 1 && lane <= OUT && c >= 0 && c < G.n;
 #pragma unroll
-            for (int o = 0; o < 5; ++o) {
-                const int d = c[a] + o - 2;
-                flat[o] = w && (d <= 0 || d >= n - 1);
-            }
-            const bool wall_m = w && c[a] == 0, wall_p = w && c[a] == n - 1;
-            // face velocities (Eq. step1): minus face between cells 1 and 2 of
-            // the five, plus face between 2 and 3
-            const double* rho = io.q[0];
-            const double* m = io.q[1 + a];
-            const double um = wall_m ? 0.0 : lm::idiv(m[id[1]] + m[id[2]], rho[id[1]] + rho[id[2]]);
-            const double up = wall_p ? 0.0 : lm::idiv(m[id[2]] + m[id[3]], rho[id[2]] + rho[id[3]]);
-            for (int q = 0; q < G.nq; ++q) {
-                const double* v = io.q[q];
-                double x[5];
-#pragma unroll
-                for (int o = 0; o < 5; ++o) x[o] = v[id[o]];
-                double sl[4];        // slopes of cells 1..4 of the five
-#pragma unroll
-                for (int o = 1; o < 4; ++o) sl[o] = flat[o] ? 0.0 : minmod(x[o] - x[o - 1], x[o + 1] - x[o]);
-                // minus face: left state from cell 1, right state from cell 2
-                const double fm = um > 0.0 ? (x[1] + 0.5 * sl[1]) * um : (x[2] - 0.5 * sl[2]) * um;
-                const double fp = up > 0.0 ? (x[2] + 0.5 * sl[2]) * up : (x[3] - 0.5 * sl[3]) * up;
-                acc[q] -= dt * (fp - fm) * G.rh[a];
-            }
+        for (int q = 0; q < NQ; ++q) {
+            const double d = xc[q] - xm[q], dn = __shfl_down_sync(~0u, d, 1);
+            const double s = flat ? 0.0 : minmod(d, dn), sm = __shfl_up_sync(~0u, s, 1);
+            const double f = face_flux(w, xm[q], sm, xc[q], s), fn = __shfl_down_sync(~0u, f, 1);
+            if (put) io.out[q][ic] = xc[q] + (f - fn);
         }
-        for (int q = 0; q < G.nq; ++q) io.out[q][idx] = acc[q];
     }
+}
+
+// The pass along y (A = 1) or z (A = 2): a thread takes L cells of a column.
+template <int A, int NQ, bool FIRST>
+__global__ void __launch_bounds__(128) k_advect_col(AdvGeo G, AdvIO io) {
+    const int q0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q0 >= G.rows) return;
+    const int col = q0 / G.inner * G.outer + q0 % G.inner;
+    const int c0 = blockIdx.y * G.L, c1 = min(c0 + G.L, G.n);
+    double xm[NQ], xc[NQ], d[NQ], s[NQ], f[NQ];
+    {
+        const int i0 = col + along(c0 - 2, G.n, G.wall) * G.stride, i1 = col + along(c0 - 1, G.n, G.wall) * G.stride,
+                  i2 = col + c0 * G.stride;
+        const bool flat = flat_at(G, c0 - 1);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            xm[q] = io.q[q][i1];
+            xc[q] = io.q[q][i2];
+            d[q] = xc[q] - xm[q];
+            s[q] = flat ? 0.0 : minmod(xm[q] - io.q[q][i0], d[q]);
+        }
+    }
+    double xn[NQ], o[NQ];                                  // the next face's loads, a face ahead
+    auto fetch = [&](int c) {
+        const int in = col + along(c + 1, G.n, G.wall) * G.stride, im = col + (c - 1) * G.stride;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            xn[q] = io.q[q][in];
+            if (!FIRST && c > c0) o[q] = io.out[q][im];
+        }
+    };
+    fetch(c0);
+    for (int c = c0; c <= c1; ++c) {                       // the minus face of cell c, the update of cell c - 1
+        const int im = col + (c - 1) * G.stride;
+        const double w = face_w(G, c, xm[0], xc[0], xm[1 + A], xc[1 + A]);
+        const bool flat = flat_at(G, c);
+        double y[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) y[q] = FIRST ? xm[q] : o[q];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const double dn = xn[q] - xc[q];
+            const double sc = flat ? 0.0 : minmod(d[q], dn);
+            const double fc = face_flux(w, xm[q], s[q], xc[q], sc);
+            if (c > c0) y[q] += f[q] - fc;
+            xm[q] = xc[q];
+            xc[q] = xn[q];
+            d[q] = dn;
+            s[q] = sc;
+            f[q] = fc;
+        }
+        if (c < c1) fetch(c + 1);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            if (c > c0) io.out[q][im] = y[q];
+    }
+}
+
+// Cells a thread of a column pass: the first face and slopes cost about one more
+// cell, so long chunks, but no longer than leaves every SM six warps (one against
+// two and four cells: 96 x 56 17, 19 and 23 us; two against four: 256^2 25 and 27;
+// nine against four: 32 x 96 x 120 132 and 150).
+int column_cells(long long N, int n) {
+    const long long l = N / (152 * 170);
+    int L = (int)(l < 1 ? 1 : (l > 16 ? 16 : l));
+    L = L < n / 65535 + 1 ? n / 65535 + 1 : L;            // (a grid holds 65535 of them)
+    const int chunks = (n + L - 1) / L;
+    return (n + chunks - 1) / chunks;
+}
+
+template <int NQ>
+void launch_advect(const int n[3], const double rh[3], const int wall[3], double dt, const AdvIO& io, cudaStream_t s) {
+    const long long N = (long long)n[0] * n[1] * n[2];
+    bool first = true;
+    for (int a = 0; a < 3; ++a) {
+        if (n[a] == 1) continue;
+        AdvGeo G{};
+        G.n = n[a];
+        G.wall = wall[a];
+        G.rows = (int)(N / n[a]);
+        G.stride = a == 0 ? 1 : (a == 1 ? n[0] : n[0] * n[1]);
+        G.inner = G.stride;
+        G.outer = a == 1 ? n[0] * n[1] : 0;
+        G.k = dt * rh[a];
+        lm::count_launches(1);
+        if (a == 0) {
+            const unsigned long long warps = ((unsigned long long)G.rows * (G.n + 3) + 28) / 29, b = (warps + 7) / 8;
+            k_advect_x<NQ><<<(unsigned)(b > 152 * 64 ? 152 * 64 : b), lm::NT, 0, s>>>(G, io);
+        } else {
+            G.L = column_cells(N, G.n);
+            const dim3 grid((unsigned)((G.rows + 127) / 128), (unsigned)((G.n + G.L - 1) / G.L));
+            if (a == 1 && first) k_advect_col<1, NQ, true><<<grid, 128, 0, s>>>(G, io);
+            else if (a == 1) k_advect_col<1, NQ, false><<<grid, 128, 0, s>>>(G, io);
+            else if (first) k_advect_col<2, NQ, true><<<grid, 128, 0, s>>>(G, io);
+            else k_advect_col<2, NQ, false><<<grid, 128, 0, s>>>(G, io);
+        }
+        first = false;
+    }
+    if (first)                                             // one cell: nothing flows
+        for (int q = 0; q < NQ; ++q) cudaMemcpyAsync(io.out[q], io.q[q], sizeof(double) * N, cudaMemcpyDeviceToDevice, s);
 }
 
 __global__ void __launch_bounds__(lm::NT) k_eos_ideal(int N, double gamma, const double* __restrict__ rho,
@@ -147,32 +247,30 @@ int lm_advect(int ndim, const int64_t n[3], const double h[3], const int bc[3], 
     for (int a = 0; a < 3; ++a)
         if (n[a] < 1 || !(h[a] > 0.0) || (bc[a] != LM_BC_PERIODIC && bc[a] != LM_BC_NEUMANN)) return LM_ERR_INVALID_ARG;
     if ((ndim == 2 && n[1] != 1) || (long long)n[0] * n[1] * n[2] >= (1LL << 31)) return LM_ERR_INVALID_ARG;
-    AdvGeo G{};
-    G.N = 1;
+    const int nn[3] = {(int)n[0], (int)n[1], (int)n[2]};
+    double rh[3];
+    int wall[3];
     for (int a = 0; a < 3; ++a) {
-        G.n[a] = (int)n[a];
-        G.wall[a] = bc[a] == LM_BC_NEUMANN;
-        G.rh[a] = 1.0 / h[a];
+        wall[a] = bc[a] == LM_BC_NEUMANN;
+        rh[a] = 1.0 / h[a];
     }
-    G.N = G.n[0] * G.n[1] * G.n[2];
-    G.stride[0] = 1;
-    G.stride[1] = G.n[0];
-    G.stride[2] = G.n[0] * G.n[1];
-    G.nq = rho_c ? 6 : 5;
-    const size_t N = (size_t)G.N;
+    const int nq = rho_c ? 6 : 5;
+    const size_t N = (size_t)nn[0] * nn[1] * nn[2];
     // the outputs must not overlap the inputs (every thread reads neighbours)
     const double* ins[MAXQ] = {rho, mom, mom + N, mom + 2 * N, e, rho_c};
     double* outs[MAXQ] = {rho_new, mom_star, mom_star + N, mom_star + 2 * N, e_star, rho_c_new};
-    for (int q = 0; q < G.nq; ++q)
-        for (int r = 0; r < G.nq; ++r)
+    for (int q = 0; q < nq; ++q)
+        for (int r = 0; r < nq; ++r)
             if (outs[q] < ins[r] + N && ins[r] < outs[q] + N) return LM_ERR_INVALID_ARG;
     AdvIO io{};
-    for (int q = 0; q < G.nq; ++q) {
+    for (int q = 0; q < nq; ++q) {
         io.q[q] = ins[q];
         io.out[q] = outs[q];
     }
-    lm::count_launches(1);
-    k_advect<<<blocks_for(G.N), lm::NT, 0, (cudaStream_t)stream>>>(G, io, dt);
+    if (nq == 6)
+        launch_advect<6>(nn, rh, wall, dt, io, (cudaStream_t)stream);
+    else
+        launch_advect<5>(nn, rh, wall, dt, io, (cudaStream_t)stream);
     return finish("lm_advect");
 }
 
