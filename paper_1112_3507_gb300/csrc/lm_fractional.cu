@@ -50,8 +50,7 @@ struct AdvIO {
 };
 
 __device__ __forceinline__ double minmod(double a, double b) {
-    return __longlong_as_double(
-        (long long)lm::minmod_bits((uint64_t)__double_as_longlong(a), (uint64_t)__double_as_longlong(b)));
+    return __longlong_as_double((long long)lm::minmod_bits(lm::dbits(a), lm::dbits(b)));
 }
 
 // offset along an axis of the cell at position d in [-2, n + 1]: wrapped on a
@@ -69,7 +68,7 @@ __device__ __forceinline__ double face_w(const AdvGeo& G, int c, double rm, doub
 }
 // (dt / h) times a quantity's flux through it: the upwind side's value at the face
 __device__ __forceinline__ double face_flux(double w, double xm, double sm, double xc, double sc) {
-    const bool up = __double_as_longlong(w) > 0;
+    const bool up = (int64_t)lm::dbits(w) > 0;
     return fma(up ? 0.5 : -0.5, up ? sm : sc, up ? xm : xc) * w;
 }
 __device__ __forceinline__ bool flat_at(const AdvGeo& G, int c) { return G.wall && (c <= 0 || c >= G.n - 1); }

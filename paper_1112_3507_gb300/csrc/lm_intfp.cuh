@@ -29,8 +29,7 @@
 // About 65 integer instructions, against seven (reciprocal) and eleven
 // (quotient) issue slots of the float64 pipe at 18.5 cycles an SM each.
 //
-// Sign, finiteness and order of float64 values are those of their bits (a zero is
-// tested by a shift: the compiler makes a float64 comparison of a masked test); a
+// Sign, finiteness and order of float64 values are those of their bits; a
 // conversion between normal float32 and float64 values shifts the mantissa.
 #pragma once
 
@@ -80,6 +79,14 @@ LM_HD int64_t idiv_core(uint64_t ma, uint64_t mb, int e, uint64_t y) {
 }
 
 #ifdef __CUDACC__
+// the bits of a computed value, opaque to the compiler, which makes float64
+// comparisons of tests on bits that it sees come from float64 arithmetic
+__device__ __forceinline__ uint64_t dbits(double v) {
+    uint64_t u;
+    asm("mov.b64 %0, %1;" : "=l"(u) : "d"(v));
+    return u;
+}
+
 __device__ __forceinline__ uint32_t idiv_seed(uint64_t m) {
     const float f = __uint_as_float(0x3f800000u | (uint32_t)(m >> 29));
     float r;
@@ -89,7 +96,7 @@ __device__ __forceinline__ uint32_t idiv_seed(uint64_t m) {
 
 // a / b, rounded to nearest
 __device__ __forceinline__ double idiv(double a, double b) {
-    const uint64_t ua = (uint64_t)__double_as_longlong(a), ub = (uint64_t)__double_as_longlong(b);
+    const uint64_t ua = dbits(a), ub = dbits(b);
     const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff, e = ea - eb + 1023;
     const uint64_t M = (1ull << 52) - 1;
     // normal operands and a result that stays normal whichever way it rounds
@@ -106,12 +113,12 @@ __device__ __forceinline__ double ircp(double b) { return idiv(1.0, b); }
 
 // v > 0 and finite
 __device__ __forceinline__ bool pos_finite(double v) {
-    return (uint64_t)(__double_as_longlong(v) - 1) < 0x7ff0000000000000ull - 1;
+    return dbits(v) - 1 < 0x7ff0000000000000ull - 1;
 }
 
 // (float)v, rounded to nearest even
 __device__ __forceinline__ float to_f32(double v) {
-    const uint64_t u = (uint64_t)__double_as_longlong(v), m = u & 0x7fffffffffffffffull;
+    const uint64_t u = dbits(v), m = u & 0x7fffffffffffffffull;
     // exponents of normal float32 values, one short of the largest so that a
     // carry is one too
     if (m - (897ull << 52) < (1149ull - 897ull + 1) << 52) {
@@ -133,13 +140,15 @@ __device__ __forceinline__ double to_f64(float v) {
 
 // v times a factor that is 2^k, or no such power (k = POW2_NONE)
 constexpr int POW2_NONE = 0x7fffffff;
+// (a call: as an inlined alternative it would be executed, predicated off, for all)
+static __device__ __noinline__ double mul_call(double v, double factor) { return v * factor; }
 __device__ __forceinline__ double mul_pow2(double v, double factor, int k) {
-    const uint64_t u = (uint64_t)__double_as_longlong(v);
+    const uint64_t u = dbits(v);
     const int e = (int)(u >> 52) & 0x7ff;
     if (k != POW2_NONE && (unsigned)(e - 1) < 2046u && (unsigned)(e + k - 1) < 2046u)
         return __longlong_as_double((long long)u + ((long long)k << 52));
     if (!(u << 1) && k != POW2_NONE) return v;
-    return v * factor;
+    return mul_call(v, factor);
 }
 #endif
 

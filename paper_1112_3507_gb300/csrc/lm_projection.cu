@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(lm::NT) k_projection_update(ProjGeo G, double 
         double div = 0.0, ugp = 0.0;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
+            const double k = 2.0 * dt * G.ih[a];
             const double* ua = uf_s + (size_t)a * N;
             double um = 0.0, mnew = m_s[(size_t)a * N + idx];
             if (ax[a].live) {
@@ -131,10 +132,9 @@ __global__ void __launch_bounds__(lm::NT) k_projection_update(ProjGeo G, double 
                 mnew -= dt * gp;                                         // Eq. momupdate
                 // step (vii) on the minus and plus faces
                 um = ax[a].wm ? 0.0
-                              : ua[idx] - lm::idiv(dt * (Pc - P[ax[a].m]) * G.ih[a] * 2.0, rn + rho_n[ax[a].m]);
+                              : ua[idx] - lm::idiv(k * (Pc - P[ax[a].m]), rn + rho_n[ax[a].m]);
                 const double up = ax[a].wp ? 0.0
-                                           : ua[ax[a].p] - lm::idiv(dt * (P[ax[a].p] - Pc) * G.ih[a] * 2.0,
-                                                                    rho_n[ax[a].p] + rn);
+                                           : ua[ax[a].p] - lm::idiv(k * (P[ax[a].p] - Pc), rho_n[ax[a].p] + rn);
                 div += (up - um) * G.ih[a];
                 ugp += lm::idiv(mnew, rn) * gp;
             }

@@ -44,7 +44,7 @@ __device__ __forceinline__ double apply64_fix(int idx, const Geo& g, const Op64&
     const bool y = g.ny > 1;
     const Nbr nx = nbr_x(idx, i, g), nz = nbr_z(idx, k, g), ny = y ? nbr_y(idx, j, g) : nx;
     const double xc = x[idx];
-    const uint64_t uc = (uint64_t)__double_as_longlong(xc);
+    const uint64_t uc = dbits(xc);
     uint64_t X[4], W[4];
     auto ld = [](const double* p, int q) { return (uint64_t)__double_as_longlong(p[q]); };
     X[0] = ld(x, nx.im), X[1] = ld(x, nx.ip), W[0] = ld(op.gx, idx), W[1] = ld(op.gx, nx.ip);
