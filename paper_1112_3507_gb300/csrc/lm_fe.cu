@@ -280,7 +280,7 @@ struct FeFlags {
 using lm::pos_finite;
 // 0, or 2^-125 < |v| < 2^126, by the bits
 __device__ __forceinline__ bool normal32(double v) {
-    const uint64_t m = (uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    const uint64_t m = lm::dbits(v) & 0x7fffffffffffffffull;
     return m << 1 == 0 || (m > (898ull << 52) && m < (1149ull << 52));
 }
 
@@ -670,6 +670,7 @@ struct lm_fe {
     double c[8] = {0};
     double kd = 0.0;           // K_ref's diagonal entry
     int faces = 1;
+    int KZ = 1;                // planes a block of the column kernel
     lm_grid* fv = nullptr;     // cell-centred grid on the same points (the preconditioner's hierarchy)
     double *ke = nullptr, *vc = nullptr, *dinv = nullptr;
     double *f = nullptr, *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
@@ -732,6 +733,23 @@ int fe_init_state(lm_fe* fe, SolveState* st, double rtol, cudaStream_t s) {
     return LM_OK;
 }
 
+// Planes a block of the column kernel marches.  Four blocks an SM are resident
+// (64 registers a thread), and every wave of them takes about its planes and two
+// more to fill the windows: the count of chunks with the least waves x (KZ + 2)
+// (256^3 solve: 20.9 ms with five chunks, 2.1 waves; 19.5 with seven, 2.95; the
+// model orders all of 2 to 19 chunks as measured).
+int fe_planes(const FeGeo& g) {
+    const long long cols = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+    long long best = 0;
+    int KZ = g.nz;
+    for (int c = 1; c <= g.nz && c <= 4 * 152; ++c) {
+        const int kz = (g.nz + c - 1) / c;
+        const long long blocks = cols * ((g.nz + kz - 1) / kz), cost = (blocks + 4 * 152 - 1) / (4 * 152) * (kz + 2);
+        if (c == 1 || (cost < best && blocks <= lm::MAX_PARTIALS)) best = cost, KZ = kz;
+    }
+    return KZ;
+}
+
 // float32 operator kernel of the given mode; dots as in fe_out
 template <int MODE, int DOTS>
 void launch_fe32_d(const lm_fe* fe, cudaStream_t s, const FeIO32& io) {
@@ -739,9 +757,7 @@ void launch_fe32_d(const lm_fe* fe, cudaStream_t s, const FeIO32& io) {
     lm::count_launches(1);
     const int bx = (fe->geo.nx + 31) / 32, by = (fe->geo.ny + 7) / 8;
     const long long cols = (long long)bx * by;
-    int chunks = (int)std::max(1LL, std::min<long long>(fe->geo.nz, (8LL * 152 + cols - 1) / cols));
-    const int KZ = (fe->geo.nz + chunks - 1) / chunks;
-    chunks = (fe->geo.nz + KZ - 1) / KZ;
+    const int KZ = fe->KZ, chunks = (fe->geo.nz + KZ - 1) / KZ;
     // one reduction partial a block: the column kernel when its blocks fit
     if (fe->geo.dim == 3 && cols * chunks <= lm::MAX_PARTIALS) {
         const dim3 grid(bx, by, chunks), block(32, 8);
@@ -1023,6 +1039,7 @@ int lm_fe_create(int ndim, const int64_t n[3], const double h[3], const int bc[3
     const double tiny = 1e-14 * std::fabs(fe->kd);
     fe->faces = (std::fabs(fe->c[1]) > tiny || std::fabs(fe->c[2]) > tiny || std::fabs(fe->c[4]) > tiny) ? 1 : 0;
     if (!fe->faces) fe->c[1] = fe->c[2] = fe->c[4] = 0.0;
+    fe->KZ = fe_planes(fe->geo);
     const size_t N = fe->N;
     int rc = lm_grid_create(ndim, n, h, bc, &fe->fv);
     double** d64[] = {&fe->ke, &fe->vc, &fe->dinv, &fe->f, &fe->x, &fe->r, &fe->p, &fe->q};
