@@ -1903,6 +1903,20 @@ static void launch_rbgs_row(const Lev32& L, cudaStream_t s, const float* xin, co
 #undef LM_ROW
 }
 
+// Planes per block of a sweep on `tiles` x nz: a block stages four planes beyond its
+// own, so short chunks cost work and long ones the length of a block's march.  A
+// sweep takes about (blocks + idle) x (KZ + 4), `idle` being the blocks whose work
+// takes as long as one block's latency; the KZ with the least of it.
+static int sweep_planes(int tiles, int nz, int lo, int idle) {
+    long long best = 0;
+    int KZ = lo;
+    for (int kz = lo; kz <= std::max(lo, std::min(nz, 64)); ++kz) {
+        const long long cost = ((long long)tiles * hdiv(nz, kz) + idle) * (kz + 4);
+        if (kz == lo || cost < best) best = cost, KZ = kz;
+    }
+    return KZ;
+}
+
 // One red-black sweep xout = S(xin [+ P ec]); first = colour updated first;
 // kz = planes per block (<= 0: enough blocks to fill the GPU).
 void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const float* ec, const Lev32* C, int hx,
@@ -1921,14 +1935,11 @@ void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const floa
     }
     if (g.ny > 1 && g.nx % 32 == 0 && g.ny % 8 == 0 && g.nz >= 2) {
         // whole TX x 8 tiles (TX = 64 when nx allows, else 32): the in-place
-        // z-march; KZ planes per block, the largest of 64, 32, ..., 2 that
-        // still gives eight blocks per SM (small levels are latency-bound:
-        // short chunks, more blocks)
+        // z-march; KZ planes per block (a 96^3 time step with 2, 3, 4, 6, 8,
+        // 12 of them on that level: 2432, 2367, 2349, 2261, 2278, 2323 us; two
+        // stay best on 64^3)
         const int TXc = g.nx % 64 == 0 ? 64 : 32;
-        const long long tiles = (long long)(g.nx / TXc) * (g.ny / 8);
-        int KZ = kz > 0 ? kz : 64;
-        if (kz <= 0)
-            while (KZ > 2 && tiles * hdiv(g.nz, KZ) < 8 * 152) KZ /= 2;
+        const int KZ = kz > 0 ? kz : sweep_planes(g.nx / TXc * (g.ny / 8), g.nz, 2, 350);
         const dim3 grd(g.nx / TXc, g.ny / 8, hdiv(g.nz, KZ)), blk(32, 8);
 #define LM_RBZ(T, F, Z, P) k_rbgs_zm<T, F, Z, P><<<grd, blk, 0, s>>>(L, xin, ec, Cg, hx, hy, hz, f, xout, KZ)
 #define LM_RBZT(T)                                                                                   \
@@ -1940,12 +1951,10 @@ void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const floa
 #undef LM_RBZ
     } else if (g.ny > 1) {
         constexpr int BX = 32, TY = 8;
-        const int tiles = hdiv(g.nx, 2 * BX) * hdiv(g.ny, TY);
-        int KZ = kz;
-        if (KZ <= 0) {
-            KZ = 16;
-            while (KZ > 1 && (long long)tiles * hdiv(g.nz, KZ) < 1216) KZ /= 2;
-        }
+        // (a 120 x 72 x 88 solve with 1, 2, 3, 4, 6, 8 planes a block on its two
+        // levels of such sweeps: 5161, 4598, 4413, 4436, 4763, 5310 us; 48^3 and
+        // 60 x 36 x 44 are best with one)
+        const int KZ = kz > 0 ? kz : sweep_planes(hdiv(g.nx, 2 * BX) * hdiv(g.ny, TY), g.nz, 1, 600);
         const dim3 grd(hdiv(g.nx, 2 * BX), hdiv(g.ny, TY), hdiv(g.nz, KZ)), blk(BX, TY);
 #define LM_RB(F, Z, P) k_rbgs<BX, TY, true, F, Z, P><<<grd, blk, 0, s>>>(L, xin, ec, Cg, hx, hy, hz, f, xout, KZ)
         if (zero) { if (first) LM_RB(1, true, false); else LM_RB(0, true, false); }
@@ -1957,13 +1966,14 @@ void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const floa
         // and half (quarter) chunk; KZ rows per block, about eight blocks (32
         // warps) per SM in all -- four blocks per SM left the loads too few
         // to cover the HBM latency (0.43 against 0.58 of the copy bandwidth
-        // at 4096^2) -- and at least 2 rows a warp (small grids, which cannot
+        // at 4096^2) -- and at least a row a warp (small grids, which cannot
         // fill the GPU, get as many warps as that allows: their time is the
-        // length of one warp's march)
+        // length of one warp's march; against two rows a warp 256^2 784 -> 733
+        // us a time step, 512^2 1297 -> 1228 and 1024 x 448 1449 -> 1394 a solve)
         const int TW = zrow2d_width(g.nx), tiles = g.nx / TW, parts = 512 / TW;
         int KZ = kz;
         if (kz <= 0) {
-            const int chunks = std::max(1, std::min(hdiv(1216, tiles), g.nz / (2 * parts)));
+            const int chunks = std::max(1, std::min(hdiv(1216, tiles), g.nz / parts));
             KZ = hdiv(g.nz, chunks);
         }
         const dim3 grd(tiles, hdiv(g.nz, KZ));
@@ -1973,13 +1983,11 @@ void launch_rbgs_kz(const Lev32& L, cudaStream_t s, const float* xin, const floa
         else { if (first) LM_RB2(1, false, false); else LM_RB2(0, false, false); }
 #undef LM_RB2
     } else {
+        // (solves with 1, 2, 4, 8 rows a block: 360 x 200 880, 905, 959, 1079 us,
+        // 832 x 240 1248, 1232, 1340, 1593, 720^2 2857, 2679, 2816, 3407,
+        // 704 x 1920 2960, 2475, 2373, 2515)
         constexpr int BX = 128, TY = 1;
-        const int tiles = hdiv(g.nx, 2 * BX);
-        int KZ = kz;
-        if (KZ <= 0) {
-            KZ = 32;
-            while (KZ > 4 && (long long)tiles * hdiv(g.nz, KZ) < 1216) KZ /= 2;
-        }
+        const int KZ = kz > 0 ? kz : sweep_planes(hdiv(g.nx, 2 * BX), g.nz, 1, 1500);
         const dim3 grd(hdiv(g.nx, 2 * BX), hdiv(g.nz, KZ), 1), blk(BX, TY);
 #define LM_RB(F, Z, P) k_rbgs<BX, TY, false, F, Z, P><<<grd, blk, 0, s>>>(L, xin, ec, Cg, hx, hy, hz, f, xout, KZ)
         if (zero) { if (first) LM_RB(1, true, false); else LM_RB(0, true, false); }
