@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(NT) k_finish_rel(double* part, int G, SolveSta
 // float32 range; it saves a float64 multiply a cell on GB300's slow float64
 // pipe); 2 scaled in float64 before rounding.
 // ZERO: x = 0 (which it sets), so r = f: a kernel of its own, since the stencil's
-// registers would leave this one, bound by memory, too few warps (256^3: 111 -> 82 us).
+// registers would leave this one, bound by memory, too few warps (256^3: 130 -> 56 us).
 template <bool FNORM, int SC, bool ZERO>
 __global__ void __launch_bounds__(NT) k_ir_residual(Geo g, Op64 op, const double* __restrict__ f,
                                                     double* __restrict__ x, float* __restrict__ r32,

@@ -21,7 +21,7 @@
 // thread marches up a chunk of a column and keeps the last face in registers;
 // along x the lanes of a warp hold successive cells and pass differences, slopes
 // and fluxes by shuffles.  The passes after the first add to the outputs.
-// Five quantities on 96^3 791 -> 234 us, on 256^2 52 -> 25 us.
+// Five quantities on 96^3 791 -> 175 us, on 256^2 52 -> 21 us.
 #include <cuda_runtime.h>
 
 #include <cstdio>

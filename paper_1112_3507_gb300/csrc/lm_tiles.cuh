@@ -110,7 +110,7 @@ __device__ __forceinline__ void assemble_range(const AsmArgs& a, int start, int 
         // 2 ulp otherwise.  The four reciprocals, the tests and the conversions
         // run on the integer pipe (lm_intfp.cuh), which leaves the float64 pipe
         // five sums and products a cell and one more per axis whose 2/h^2 is no
-        // power of two: 256^3 1062 -> 439 us
+        // power of two: 256^3 1062 -> 381 to 456 us
         const double gxm =
             face_minus(i, g.nx, g.bcx) ? mul_pow2(ircp(rn + rho_new[nbr_x(idx, i, g).im]), c2x, a.kx) : 0.0;
         const double gym =
