@@ -41,7 +41,7 @@ struct AdvGeo {
     int rows;                 // columns of the axis: N / n
     int inner, outer;         // column q starts at (q / inner) outer + q % inner
     int L;                    // cells a thread (y and z)
-    double k;                 // dt / h
+    double dt, rh;            // rh = 1 / h
 };
 
 struct AdvIO {
@@ -62,11 +62,11 @@ __device__ __forceinline__ int along(int d, int n, int wall) {
     return d;
 }
 
-// (dt / h) u of the minus face of the cell at position c (Eq. step1), cells m and c
+// dt u of the minus face of the cell at position c (Eq. step1), cells m and c
 __device__ __forceinline__ double face_w(const AdvGeo& G, int c, double rm, double rc, double mm, double mc) {
-    return G.wall && (c == 0 || c == G.n) ? 0.0 : G.k * lm::idiv(mm + mc, rm + rc);
+    return G.wall && (c == 0 || c == G.n) ? 0.0 : G.dt * lm::idiv(mm + mc, rm + rc);
 }
-// (dt / h) times a quantity's flux through it: the upwind side's value at the face
+// dt times a quantity's flux through it: the upwind side's value at the face
 __device__ __forceinline__ double face_flux(double w, double xm, double sm, double xc, double sc) {
     const bool up = (int64_t)lm::dbits(w) > 0;
     return fma(up ? 0.5 : -0.5, up ? sm : sc, up ? xm : xc) * w;
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(lm::NT) k_advect_x(AdvGeo G, AdvIO io) {
             const double d = xc[q] - xm[q], dn = __shfl_down_sync(~0u, d, 1);
             const double s = flat ? 0.0 : minmod(d, dn), sm = __shfl_up_sync(~0u, s, 1);
             const double f = face_flux(w, xm[q], sm, xc[q], s), fn = __shfl_down_sync(~0u, f, 1);
-            if (put) io.out[q][ic] = xc[q] + (f - fn);
+            if (put) io.out[q][ic] = fma(G.rh, f - fn, xc[q]);
         }
     }
 }
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(128) k_advect_col(AdvGeo G, AdvIO io) {
             const double dn = xn[q] - xc[q];
             const double sc = flat ? 0.0 : minmod(d[q], dn);
             const double fc = face_flux(w, xm[q], s[q], xc[q], sc);
-            if (c > c0) y[q] += f[q] - fc;
+            if (c > c0) y[q] = fma(G.rh, f[q] - fc, y[q]);
             xm[q] = xc[q];
             xc[q] = xn[q];
             d[q] = dn;
@@ -186,7 +186,8 @@ void launch_advect(const int n[3], const double rh[3], const int wall[3], double
         G.stride = a == 0 ? 1 : (a == 1 ? n[0] : n[0] * n[1]);
         G.inner = G.stride;
         G.outer = a == 1 ? n[0] * n[1] : 0;
-        G.k = dt * rh[a];
+        G.dt = dt;
+        G.rh = rh[a];
         lm::count_launches(1);
         if (a == 0) {
             const unsigned long long warps = ((unsigned long long)G.rows * (G.n + 3) + 28) / 29, b = (warps + 7) / 8;
