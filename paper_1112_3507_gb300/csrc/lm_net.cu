@@ -19,6 +19,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -884,8 +885,11 @@ __global__ void __launch_bounds__(256) k_pool_bwd(const float* __restrict__ g, c
 }
 #undef LM_PIXELS
 
-// loss = mean((y - t)^2), gy = 2 (y - t) / n (deterministic grid reduction;
-// one block over all pixels had taken 2.1 ms for 16 images of 256^2)
+// gy = 2 (y - t) / n and, with LOSS, loss = mean((y - t)^2) (deterministic grid
+// reduction; one block over all pixels had taken 2.1 ms for 16 images of 256^2)
+constexpr int LOSS_BLOCKS = 2 * 152;
+constexpr int LOSS_WORDS = LOSS_BLOCKS + 2;        // the loss, the blocks' sums, the arrival counter
+template <bool LOSS>
 __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const float* __restrict__ t,
                                              float* __restrict__ gy, long long n, Red red) {
     __shared__ double sm[32];
@@ -894,8 +898,9 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const 
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
         const float d = y[i] - t[i];
         gy[i] = 2.f * d / (float)n;
-        ff_add_prod(acc, d, d);
+        if (LOSS) ff_add_prod(acc, d, d);
     }
+    if (!LOSS) return;
     v[0] = ff_value(acc);
     const int sl[1] = {0};
     if (grid_reduce<1>(v, red, sl, sm) && threadIdx.x == 0) red.scal[0] /= (double)n;
@@ -954,6 +959,7 @@ struct lm_net {
     size_t part_n = 0;
     double* sums = nullptr;         // per-channel block sums of the backward pass
     double* dloss = nullptr;        // loss, its block sums and their arrival counter
+    std::mutex loss_mu;             // held by a call that uses them, until it has read the loss
     int adam_t = 0;
 };
 
@@ -1256,8 +1262,9 @@ int net_create(const int ch[4], lm_net** out) {
         np += (size_t)(c.cin + 15) / 16 * 9 * c.cout * 16;
         npt += (size_t)(c.cout + 15) / 16 * 9 * c.cin * 16;
     }
-    if (cudaMalloc(&N->wp, np * 2) || cudaMalloc(&N->wpt, npt * 2) || cudaMalloc(&N->master, n * 4) || cudaMalloc(&N->grad, n * 4) || cudaMalloc(&N->m, n * 4) ||
-        cudaMalloc(&N->v, n * 4) || cudaMalloc(&N->wb, n * 2) || cudaMalloc(&N->wt, n * 2)) {
+    if (cudaMalloc(&N->wp, np * 2) || cudaMalloc(&N->wpt, npt * 2) || cudaMalloc(&N->master, n * 4) ||
+        cudaMalloc(&N->grad, n * 4) || cudaMalloc(&N->m, n * 4) || cudaMalloc(&N->v, n * 4) ||
+        cudaMalloc(&N->wb, n * 2) || cudaMalloc(&N->wt, n * 2) || cudaMalloc(&N->dloss, LOSS_WORDS * 8)) {
         net_destroy(N);
         return LM_ERR_OUT_OF_MEMORY;
     }
@@ -1266,6 +1273,12 @@ int net_create(const int ch[4], lm_net** out) {
     cudaMemset(N->m, 0, n * 4);
     cudaMemset(N->v, 0, n * 4);
     cudaMemset(N->wb, 0, n * 2);
+    cudaMemset(N->dloss, 0, LOSS_WORDS * 8);
+    // the clears run on the default stream, which a caller's stream need not wait for
+    if (cudaDeviceSynchronize() != cudaSuccess) {
+        net_destroy(N);
+        return LM_ERR_CUDA;
+    }
     *out = N;
     return LM_OK;
 }
@@ -1459,17 +1472,19 @@ int lm_net_backward(lm_net* N, const float* gy, void* stream) {
 int lm_net_mse(lm_net* N, const float* y, const float* t, float* gy, long long n, double* loss, void* stream) {
     if (!N || !y || !t || !gy || n < 1) return LM_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int nb = (int)std::max(1LL, std::min(2LL * 152, (n + 1023) / 1024));
-    if (!N->dloss) {                               // the loss, up to 304 block sums, and the arrival counter
-        NCK(cudaMalloc(&N->dloss, sizeof(double) * 306));
-        NCK(cudaMemset(N->dloss, 0, sizeof(double) * 306));
-    }
+    const int nb = (int)std::max<long long>(1, std::min<long long>(LOSS_BLOCKS, (n + 1023) / 1024));
     count_launches(1);
-    k_mse<<<nb, 256, 0, s>>>(y, t, gy, n, Red{N->dloss + 1, N->dloss, (unsigned int*)(N->dloss + 305)});
-    if (loss) {
-        NCK(cudaMemcpyAsync(loss, N->dloss, sizeof(double), cudaMemcpyDeviceToHost, s));
-        NCK(cudaStreamSynchronize(s));
+    if (!loss) {
+        k_mse<false><<<nb, 256, 0, s>>>(y, t, gy, n, Red{});
+        return cudaGetLastError() == cudaSuccess ? LM_OK : LM_ERR_CUDA;
     }
+    // one loss at a time: calls on other streams would share the counter
+    std::lock_guard<std::mutex> lk(N->loss_mu);
+    k_mse<true><<<nb, 256, 0, s>>>(
+        y, t, gy, n, Red{N->dloss + 1, N->dloss, (unsigned int*)(N->dloss + 1 + LOSS_BLOCKS)});
+    NCK(cudaGetLastError());
+    NCK(cudaMemcpyAsync(loss, N->dloss, sizeof(double), cudaMemcpyDeviceToHost, s));
+    NCK(cudaStreamSynchronize(s));
     return LM_OK;
 }
 
