@@ -386,8 +386,9 @@ bool conv3_mma(const void* in, int Cin, const bf16* Wp, const float* bias, void*
     return true;
 }
 
-// The weights' derived layouts, formed once after they change, all layers in
-// one launch:
+// The weights' derived layouts, all layers in one launch, formed by the calls
+// that change the weights, on their stream, so that a forward or backward pass
+// captured in a graph reads the weights of the time it is replayed:
 //   wt[t][co][ci] = w[8 - t][ci][co]: the backward-data convolution is a
 //     forward convolution of the output gradient with these weights;
 //   wp[c][t][co][16]: input channels 16 c .. 16 c + 15 (zero past the last) of
@@ -944,7 +945,6 @@ struct lm_net {
     bf16 *wb = nullptr, *wt = nullptr;   // BF16 weights and their flipped transposes
     bf16 *wp = nullptr, *wpt = nullptr;  // the same as the tensor-core convolutions stage them
     lm::PrepTable prep{};
-    bool prepared = false;               // wt, wp, wpt are those of the current weights
     // activations (bf16) and gradients (float) for batch x H x W
     int B = 0, H = 0, W = 0;        // the shape the buffers hold (B images at most)
     int Bf = 0;                     // images of the last forward pass
@@ -1111,12 +1111,10 @@ void mask_bias(lm_net* N, const lm_net::Conv& c, float* g, const bf16* act, long
 
 namespace lm {
 
-// the derived layouts of the weights, if they changed since they were formed
+// the derived layouts of the weights, after every change of them
 void prepare_weights(lm_net* N, cudaStream_t s) {
-    if (N->prepared) return;
     count_launches(1);
     k_prep_weights<<<dim3(32, (unsigned)N->convs.size()), 256, 0, s>>>(N->prep, N->wb, N->wt, N->wp, N->wpt);
-    N->prepared = true;
 }
 
 void net_destroy(lm_net* N);
@@ -1127,7 +1125,6 @@ int net_forward(lm_net* N, const float* xin, float* yout, int B, int H, int W, c
     if (rc) return rc;
     N->Bf = B;
     const long long P0 = (long long)B * H * W;
-    prepare_weights(N, s);
     count_launches(1);
     k_to_bf16<<<blocks_for(P0 * N->cin), 256, 0, s>>>(xin, N->x, P0 * N->cin);
     for (int l = 0; l < 4; ++l) {
@@ -1170,7 +1167,6 @@ int net_backward(lm_net* N, const float* gy, cudaStream_t s) {
     if (int rc = ensure_grads(N)) return rc;
     const int B = N->Bf, H = N->H, W = N->W;     // the images of the last forward pass
     const long long P0 = (long long)B * H * W;
-    prepare_weights(N, s);
     {   // output layer, and D_0's masked gradient with its bias gradient
         const int C = N->ch[0], V = chan_width(C), nb = elt_blocks(P0, C, V);
         const size_t n = (size_t)nb * C;
@@ -1273,6 +1269,9 @@ int net_create(const int ch[4], lm_net** out) {
     cudaMemset(N->m, 0, n * 4);
     cudaMemset(N->v, 0, n * 4);
     cudaMemset(N->wb, 0, n * 2);
+    cudaMemset(N->wt, 0, n * 2);
+    cudaMemset(N->wp, 0, np * 2);
+    cudaMemset(N->wpt, 0, npt * 2);
     cudaMemset(N->dloss, 0, LOSS_WORDS * 8);
     // the clears run on the default stream, which a caller's stream need not wait for
     if (cudaDeviceSynchronize() != cudaSuccess) {
@@ -1304,10 +1303,10 @@ int net_set_params(lm_net* N, const float* host, int n) {
     NCK(cudaMemcpy(N->master, host, sizeof(float) * n, cudaMemcpyHostToDevice));
     count_launches(1);
     k_to_bf16<<<blocks_for(n), 256>>>(N->master, N->wb, n);
+    prepare_weights(N, nullptr);
     NCK(cudaMemset(N->m, 0, sizeof(float) * n));
     NCK(cudaMemset(N->v, 0, sizeof(float) * n));
     N->adam_t = 0;
-    N->prepared = false;
     NCK(cudaDeviceSynchronize());
     return LM_OK;
 }
@@ -1491,11 +1490,11 @@ int lm_net_mse(lm_net* N, const float* y, const float* t, float* gy, long long n
 int lm_net_adam(lm_net* N, float lr, float b1, float b2, float eps, void* stream) {
     if (!N || !(lr > 0.f)) return LM_ERR_INVALID_ARG;
     const int t = ++N->adam_t;
-    N->prepared = false;
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
     count_launches(1);
     k_adam<<<blocks_for(N->nparams), 256, 0, (cudaStream_t)stream>>>(N->master, N->grad, N->m, N->v, N->wb,
                                                                      N->nparams, lr, b1, b2, eps, c1, c2);
+    lm::prepare_weights(N, (cudaStream_t)stream);
     return cudaGetLastError() == cudaSuccess ? LM_OK : LM_ERR_CUDA;
 }
 
