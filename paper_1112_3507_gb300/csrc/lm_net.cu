@@ -672,18 +672,54 @@ __global__ void k_conv1_fwd(const bf16* __restrict__ d, const float* __restrict_
 // layer's ReLU and summed per channel (the bias gradient).  Those sums ride on
 // the pass that writes the gradient: a thread keeps V consecutive channels
 // over its share of the pixels (16-byte accesses for V = 8) and sums them as
-// float pairs (FF: TwoSum, about 48 bits over the few dozen pixels of a
-// thread), then blocks and the final kernel add in float64, in a fixed order.
-// HBM-bound.  One pass per channel and block (a block a channel, each reading
-// every pixel) had taken 4.2 ms of a 13.6 ms gradient of 16 images of 256^2.
+// three floats (TwoSum twice: exact but for a float's rounding of errors of
+// errors, 2^-72), then blocks and the final kernel add in float64, in a fixed
+// order.  HBM-bound; a float64 addition a term, at 18.5 cycles an SM, made the
+// gradient of 16 images of 256^2 350 us longer.  One pass per channel and
+// block (a block a channel, each reading every pixel) had taken 4.2 ms of a
+// 13.6 ms gradient of those images.
 constexpr int ELT_BLOCKS = 4 * 152;
 
 template <int V>
+struct FVec;
+template <int V>
+__device__ __forceinline__ FVec<V> ldf(const float* p);
+
+__device__ __forceinline__ float two_sum(float& s, float x) {      // s + x = (new s) + the returned error
+    const float t = __fadd_rn(s, x), bx = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bx)), __fsub_rn(x, bx));
+    s = t;
+    return e;
+}
+template <int V>
 struct ChanSum {                    // per-channel sums of a thread
-    FF s[V];
+    float a[V], b[V], c[V];
     __device__ __forceinline__ ChanSum() {
 #pragma unroll
-        for (int v = 0; v < V; ++v) s[v] = FF{0.f, 0.f};
+        for (int v = 0; v < V; ++v) a[v] = b[v] = c[v] = 0.f;
+    }
+    __device__ __forceinline__ void add(int v, float x) {
+        c[v] = __fadd_rn(c[v], two_sum(b[v], two_sum(a[v], x)));
+    }
+    // The totals in float64 of the terms that the thread has stored in out at
+    // p0, p0 + step, ... < P of C channels.  A sum that left float32's range on
+    // the way, or met an infinity or NaN, is formed again from them.
+    __device__ __forceinline__ void totals(double (&t)[V], const float* out, long long p0, long long step, long long P,
+                                           int C) const {
+        bool lost = false;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            lost |= !isfinite(a[v]);
+            t[v] = to_f64(a[v]) + (to_f64(b[v]) + to_f64(c[v]));
+        }
+        if (!lost) return;
+#pragma unroll
+        for (int v = 0; v < V; ++v) t[v] = 0.0;
+        for (long long p = p0; p < P; p += step) {
+            const FVec<V> x = ldf<V>(out + p * C);
+#pragma unroll
+            for (int v = 0; v < V; ++v) t[v] += (double)x.v[v];
+        }
     }
 };
 
@@ -692,13 +728,13 @@ struct ChanSum {                    // per-channel sums of a thread
 // none).  256 / C threads share a channel's additions (with one thread a group
 // their float64 latencies were two thirds of a pass).
 template <int V>
-__device__ __forceinline__ void chan_store(const ChanSum<V>& a, int C, int G, int nth, double* __restrict__ part,
+__device__ __forceinline__ void chan_store(const double (&a)[V], int C, int G, int nth, double* __restrict__ part,
                                            double* sm /* 256 V */) {
     const int tid = threadIdx.x;
     __syncthreads();
     if (tid < nth)
 #pragma unroll
-        for (int v = 0; v < V; ++v) sm[v * 256 + tid] = ff_value(a.s[v]);
+        for (int v = 0; v < V; ++v) sm[v * 256 + tid] = a[v];
     __syncthreads();
     const int parts = 256 / C, o = tid % C, k = tid / C;
     double t = 0.0;
@@ -747,17 +783,25 @@ __device__ __forceinline__ BVec<V> ldb(const bf16* p) {
     return *reinterpret_cast<const BVec<V>*>(p);
 }
 
-// The pixel loop of the kernels below: thread's channel group and pixels.
+// The pixel loop of the kernels below: thread's channel group and pixels.  (Their
+// grids have up to four blocks an SM, which their registers must leave room for.)
 #define LM_PIXELS(V, C, P)                                                        \
     const int G = (C) / (V), nth = 256 / G * G, tid = threadIdx.x;                \
     const int c0 = (tid % G) * (V);                                               \
     const long long step = (long long)gridDim.x * (nth / G);                      \
-    if (tid < nth)                                                                \
-        for (long long p = (long long)blockIdx.x * (nth / G) + tid / G; p < (P); p += step)
+    const long long p0 = tid < nth ? (long long)blockIdx.x * (nth / G) + tid / G : (P); \
+    for (long long p = p0; p < (P); p += step)
+// ... and the sums s of what it stored in `out`, through the block into part.
+#define LM_SUMS(V, s, out, C, P, part)                                            \
+    do {                                                                          \
+        double t_[V];                                                             \
+        (s).totals(t_, (out) + c0, p0, step, P, C);                               \
+        chan_store<V>(t_, C, G, nth, part, sm);                                   \
+    } while (0)
 
 // g *= (act > 0); bias sums of the masked g
 template <int V>
-__global__ void __launch_bounds__(256) k_mask_bias(float* __restrict__ g, const bf16* __restrict__ act, int C,
+__global__ void __launch_bounds__(256, 4) k_mask_bias(float* __restrict__ g, const bf16* __restrict__ act, int C,
                                                    long long P, double* __restrict__ part) {
     __shared__ double sm[256 * V];
     ChanSum<V> s;
@@ -768,47 +812,48 @@ __global__ void __launch_bounds__(256) k_mask_bias(float* __restrict__ g, const 
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             if (!(__bfloat162float(a.v[v]) > 0.f)) x.v[v] = 0.f;
-            ff_add(s.s[v], x.v[v]);
+            s.add(v, x.v[v]);
         }
         *reinterpret_cast<FVec<V>*>(g + i) = x;
     }
-    chan_store<V>(s, C, G, nth, part, sm);
+    LM_SUMS(V, s, g, C, P, part);
 }
 
 // The output layer's backward: gd = gy O masked by d > 0 with its bias sums
 // (the layer below), dO = sum_p d gy, do = sum_p gy (part: three arrays of
 // blocks x C, blocks x C and blocks x 1).
 template <int V>
-__global__ void __launch_bounds__(256) k_conv1_bwd(const bf16* __restrict__ d, const float* __restrict__ gy,
+__global__ void __launch_bounds__(256, 4) k_conv1_bwd(const bf16* __restrict__ d, const float* __restrict__ gy,
                                                    const float* __restrict__ O, float* __restrict__ gd, int C,
                                                    long long P, double* __restrict__ part) {
     __shared__ double sm[256 * V];
-    ChanSum<V> sb, sw;
-    ChanSum<1> sg;
+    ChanSum<V> sb;
+    double sw[V], sg = 0.0;             // products: in float64, where they neither over- nor underflow
     float o[V];
     const int G0 = C / V;
 #pragma unroll
-    for (int v = 0; v < V; ++v) o[v] = O[(threadIdx.x % G0) * V + v];
+    for (int v = 0; v < V; ++v) o[v] = O[(threadIdx.x % G0) * V + v], sw[v] = 0.0;
     LM_PIXELS(V, C, P) {
         const size_t i = p * C + c0;
         const BVec<V> a = ldb<V>(d + i);
         const float y = gy[p];
+        const double yd = to_f64(y);
         FVec<V> x;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const float av = __bfloat162float(a.v[v]);
             x.v[v] = av > 0.f ? y * o[v] : 0.f;
-            ff_add(sb.s[v], x.v[v]);
-            ff_add_prod(sw.s[v], av, y);
+            sb.add(v, x.v[v]);
+            sw[v] = fma(to_f64(av), yd, sw[v]);
         }
-        if (c0 == 0) ff_add(sg.s[0], y);
+        if (c0 == 0) sg += yd;
         *reinterpret_cast<FVec<V>*>(gd + i) = x;
     }
     const size_t n = (size_t)gridDim.x * C;
-    chan_store<V>(sb, C, G, nth, part, sm);
+    LM_SUMS(V, sb, gd, C, P, part);
     chan_store<V>(sw, C, G, nth, part + n, sm);
     __syncthreads();
-    sm[tid] = tid < nth && c0 == 0 ? ff_value(sg.s[0]) : 0.0;
+    sm[tid] = tid < nth && c0 == 0 ? sg : 0.0;
     __syncthreads();
     if (tid == 0) {
         double t = 0.0;
@@ -832,7 +877,7 @@ __global__ void k_cat_skip(const float* __restrict__ gcat, float* __restrict__ g
 // The upsampled half: gd = up_bwd(gcat[..., :Cu]) (sum over the four fine
 // pixels) at half resolution, masked by act > 0, with its bias sums.
 template <int V>
-__global__ void __launch_bounds__(256) k_up_bwd(const float* __restrict__ gcat, const bf16* __restrict__ act,
+__global__ void __launch_bounds__(256, 4) k_up_bwd(const float* __restrict__ gcat, const bf16* __restrict__ act,
                                                 float* __restrict__ gd, int Ho, int Wo, int Cu, int Cs, long long P,
                                                 double* __restrict__ part) {
     __shared__ double sm[256 * V];
@@ -851,17 +896,17 @@ __global__ void __launch_bounds__(256) k_up_bwd(const float* __restrict__ gcat, 
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             x.v[v] = __bfloat162float(a.v[v]) > 0.f ? (a0.v[v] + a1.v[v]) + (a2.v[v] + a3.v[v]) : 0.f;
-            ff_add(s.s[v], x.v[v]);
+            s.add(v, x.v[v]);
         }
         *reinterpret_cast<FVec<V>*>(gd + p * Cu + c0) = x;
     }
-    chan_store<V>(s, Cu, G, nth, part, sm);
+    LM_SUMS(V, s, gd, Cu, P, part);
 }
 
 // gacc += pool_bwd(g) (each fine pixel receives a quarter of its parent's
 // gradient), masked by act > 0, with its bias sums.
 template <int V>
-__global__ void __launch_bounds__(256) k_pool_bwd(const float* __restrict__ g, const bf16* __restrict__ act,
+__global__ void __launch_bounds__(256, 4) k_pool_bwd(const float* __restrict__ g, const bf16* __restrict__ act,
                                                   float* __restrict__ gacc, int H, int Wd, int C, long long P,
                                                   double* __restrict__ part) {
     __shared__ double sm[256 * V];
@@ -878,13 +923,14 @@ __global__ void __launch_bounds__(256) k_pool_bwd(const float* __restrict__ g, c
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             t.v[v] = __bfloat162float(a.v[v]) > 0.f ? fmaf(0.25f, q.v[v], t.v[v]) : 0.f;
-            ff_add(s.s[v], t.v[v]);
+            s.add(v, t.v[v]);
         }
         *reinterpret_cast<FVec<V>*>(gacc + i) = t;
     }
-    chan_store<V>(s, C, G, nth, part, sm);
+    LM_SUMS(V, s, gacc, C, P, part);
 }
 #undef LM_PIXELS
+#undef LM_SUMS
 
 // gy = 2 (y - t) / n and, with LOSS, loss = mean((y - t)^2) (deterministic grid
 // reduction; one block over all pixels had taken 2.1 ms for 16 images of 256^2)
@@ -895,14 +941,15 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const 
                                              float* __restrict__ gy, long long n, Red red) {
     __shared__ double sm[32];
     double v[1] = {0.0};
-    FF acc{0.f, 0.f};
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
         const float d = y[i] - t[i];
         gy[i] = 2.f * d / (float)n;
-        if (LOSS) ff_add_prod(acc, d, d);
+        if (LOSS) {
+            const double dd = to_f64(d);
+            v[0] = fma(dd, dd, v[0]);
+        }
     }
     if (!LOSS) return;
-    v[0] = ff_value(acc);
     const int sl[1] = {0};
     if (grid_reduce<1>(v, red, sl, sm) && threadIdx.x == 0) red.scal[0] /= (double)n;
 }
@@ -1084,18 +1131,26 @@ void conv_bwd_w(lm_net* N, const lm_net::Conv& c, const bf16* act, const float* 
     k_reduce_groups<<<(n + 31) / 32, dim3(32, 8), 0, s>>>(N->part, groups, n, N->grad + c.w);
 }
 
-// V consecutive channels a thread: the widest that divides C (and C2)
-int chan_width(int C, int C2 = 0) { return C % 8 == 0 && C2 % 8 == 0 ? 8 : (C % 4 == 0 && C2 % 4 == 0 ? 4 : 1); }
+// V consecutive channels a thread: the widest that divides C (and C2); four at
+// most in the passes that would spill with eight in the registers that four
+// blocks an SM leave a thread
+int chan_width(int C, int C2 = 0, int most = 8) {
+    return most >= 8 && C % 8 == 0 && C2 % 8 == 0 ? 8 : (C % 4 == 0 && C2 % 4 == 0 ? 4 : 1);
+}
 // blocks of a pixel pass over P pixels of C channels, V a thread
 int elt_blocks(long long P, int C, int V) {
     const long long per = 256 / (C / V);
     return (int)std::max(1LL, std::min<long long>(ELT_BLOCKS, (P + per - 1) / per));
 }
-#define LM_BY_WIDTH(V, CALL)                       \
-    do {                                           \
+#define LM_BY_WIDTH4(V, CALL)                              \
+    do {                                                   \
+        if ((V) == 4) { constexpr int W_ = 4; CALL; }      \
+        else { constexpr int W_ = 1; CALL; }               \
+    } while (0)
+#define LM_BY_WIDTH(V, CALL)                               \
+    do {                                                   \
         if ((V) == 8) { constexpr int W_ = 8; CALL; }      \
-        else if ((V) == 4) { constexpr int W_ = 4; CALL; } \
-        else { constexpr int W_ = 1; CALL; }       \
+        else LM_BY_WIDTH4(V, CALL);                        \
     } while (0)
 
 // g *= (act > 0), and the bias gradient of conv c (whose output gradient g is)
@@ -1168,10 +1223,10 @@ int net_backward(lm_net* N, const float* gy, cudaStream_t s) {
     const int B = N->Bf, H = N->H, W = N->W;     // the images of the last forward pass
     const long long P0 = (long long)B * H * W;
     {   // output layer, and D_0's masked gradient with its bias gradient
-        const int C = N->ch[0], V = chan_width(C), nb = elt_blocks(P0, C, V);
+        const int C = N->ch[0], V = chan_width(C, 0, 4), nb = elt_blocks(P0, C, V);
         const size_t n = (size_t)nb * C;
         count_launches(2);
-        LM_BY_WIDTH(V, (k_conv1_bwd<W_><<<nb, 256, 0, s>>>(N->d[0], gy, N->master + N->oW, N->gd0, C, P0, N->sums)));
+        LM_BY_WIDTH4(V, (k_conv1_bwd<W_><<<nb, 256, 0, s>>>(N->d[0], gy, N->master + N->oW, N->gd0, C, P0, N->sums)));
         k_chan_final<<<dim3(C, 3), 128, 0, s>>>(ChanOut{N->sums, N->grad + N->convs[13].b, C},
                                                ChanOut{N->sums + n, N->grad + N->oW, C},
                                                ChanOut{N->sums + 2 * n, N->grad + N->ob, 1}, nb);
@@ -1189,14 +1244,14 @@ int net_backward(lm_net* N, const float* gy, cudaStream_t s) {
         conv_bwd_data(N, Cc, N->gbuf1, N->gbuf2, B, Hl, Wl, s);          // g of cat
         // the skip half waits for the encoder's own gradient; the upsampled
         // half goes down masked by d_{l+1} (d_3 = e_3), the next layer's g
-        const int V = chan_width(cu, cl), nb = elt_blocks(Pl / 4, cu, V);
+        const int V = chan_width(cu, cl), Vu = chan_width(cu, cl, 4), nb = elt_blocks(Pl / 4, cu, Vu);
         const bf16* below = l < 2 ? N->d[l + 1] : N->e[3];
         const lm_net::Conv& next = N->convs[l < 2 ? k - 1 : 7];
         float* gn = l < 2 ? N->gdl[l + 1] : N->genc[3];
         const ChanOut o{N->sums, N->grad + next.b, cu};
         count_launches(3);
         LM_BY_WIDTH(V, (k_cat_skip<W_><<<blocks_for(Pl * (cl / W_)), 256, 0, s>>>(N->gbuf2, N->genc[l], Pl, cu, cl)));
-        LM_BY_WIDTH(V, (k_up_bwd<W_><<<nb, 256, 0, s>>>(N->gbuf2, below, gn, Hl / 2, Wl / 2, cu, cl, Pl / 4, N->sums)));
+        LM_BY_WIDTH4(Vu, (k_up_bwd<W_><<<nb, 256, 0, s>>>(N->gbuf2, below, gn, Hl / 2, Wl / 2, cu, cl, Pl / 4, N->sums)));
         k_chan_final<<<dim3(cu, 1), 128, 0, s>>>(o, o, o, nb);
         gd = gn;
     }

@@ -1,0 +1,80 @@
+"""The network's float64 sums at the ends of float32's range: losses and bias
+gradients whose terms or partial sums no float32 holds, and infinities."""
+import os
+
+import numpy as np
+import pytest
+
+from oracle import unet as U
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def lm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1112_3507_gb300 import build as B
+    if not os.path.exists(B.LIB) or any(os.path.getmtime(s) > os.path.getmtime(B.LIB) for s in B.sources()):
+        B.build()
+    from paper_1112_3507_gb300 import lowmach
+    return lowmach
+
+
+# A sum of n positive terms in float64: a thread's few dozen, a tree of eight
+# steps in a block and one over the blocks stay below 64 roundings of 2^-53.
+@pytest.mark.parametrize("n", [7, 300007])
+@pytest.mark.parametrize("scale", [1e-30, 1e-22, 1.0, 1e25, 1e38])
+def test_loss(lm, n, scale):
+    rng = np.random.default_rng(n)
+    y, t = ((0.5 + rng.random(n)) * s * scale for s in (1.0, -1.0))
+    y, t = y.astype(np.float32), t.astype(np.float32)
+    d = (y - t).astype(np.float64)
+    net = lm.Net((4, 8, 8, 8))
+    yd, td = torch.as_tensor(y, device="cuda"), torch.as_tensor(t, device="cuda")
+    want = np.mean(d * d)
+    assert abs(net.mse(yd, td, torch.empty_like(yd)) - want) <= 64 * 2.0 ** -53 * want
+    net.close()
+
+
+def _net(lm, ch):
+    """D0 passes its channels through, C0 the sum of the upsampled and the skip ones; the other convolutions give their bias, 1."""
+    P = U.init_params(np.random.default_rng(0), cin=3, ch=ch)
+    for k, v in P.items():
+        v[:] = 1.0 if v.ndim == 1 or k == "O" else 0.0
+    for c in range(ch[0]):
+        P["D0"][1, 1, c, c] = P["C0"][1, 1, c, c] = P["C0"][1, 1, ch[1] + c, c] = 1.0
+    net = lm.Net(ch)
+    net.set_params(U.flat_params(P, 3, ch))
+    return net
+
+
+def _grads(lm, ch, n, gy):
+    net = _net(lm, ch)
+    net.forward(torch.zeros(3 * n * n, device="cuda"), torch.empty(n * n, device="cuda"), 1, n, n)
+    net.backward(torch.as_tensor(gy, device="cuda"))
+    g = U.unflat_params(net.grads(), 3, ch)
+    net.close()
+    return g
+
+
+# Gradients of 2^e, the first half of the pixels positive, the second negative
+# and the last zero: the sum is 2^e, and a thread's share of either half is
+# past float32's range.  (Where 2^125 is, d1's four fine pixels add up to 2^127;
+# 2^127 there would not be a float32, nor what the encoder below gets from it.)
+@pytest.mark.parametrize("names,n,e", [(("o", "d0", "c0"), 1024, 127), (("o", "d0", "c0", "b0", "d1"), 2048, 125)])
+def test_bias_gradients_past_float32(lm, names, n, e):
+    gy = np.full(n * n, 2.0 ** e, dtype=np.float32)
+    gy[n * n // 2:] *= -1
+    gy[-1] = 0.0
+    g = _grads(lm, (8, 8, 8, 8), n, gy)
+    for k in names:
+        assert np.all(g[k] == 2.0 ** e), k
+
+
+def test_infinite_gradient(lm):
+    gy = np.ones(512 * 512, dtype=np.float32)
+    gy[77] = np.inf
+    g = _grads(lm, (8, 8, 8, 8), 512, gy)
+    assert np.all(g["o"] == np.inf) and np.all(g["d0"] == np.inf)
