@@ -427,15 +427,20 @@ __global__ void k_prep_weights(PrepTable T, const bf16* __restrict__ w, bf16* __
 // tiles; as a GEMM, M = input channels, N = output channels, K = pixels, one
 // accumulator per tap, warp w taking the tile's pixel row w.  The input is
 // BF16; the float32 gradient is cut into three BF16 parts of 8 significant
-// bits each, which add up to it exactly, so each product of the sum is formed
-// without error in the FP32 accumulator's inputs.  An accumulator takes 3
-// steps a tile over at most a few dozen tiles, is added over the warps in
-// float32 and over the groups as float pairs (k_reduce_groups): the result is
-// closer to the float64 sum than the serial FP32 sums over 4096 pixels of the
-// FP32 kernel it replaced (4e-7 against 1e-6 over 2 x 256^2 pixels).  Both operands lie in shared memory pixel
-// by pixel, so fragments are read transposed (ldmatrix.trans), a tap being a
-// shift of the pixel rows; the next tile's loads fly while one is multiplied.
-// 16 images of 256^2, all layers: 3.6 ms in FP32, 0.80 ms here.
+// bits each, which add up to it exactly (above 2^-109, where no part is
+// subnormal), so each product of the sum is formed without error.  The tensor
+// cores cut an accumulator's sum off instead of rounding it, a bias that grows
+// with every step: a tile's sums therefore start at zero, smallest parts
+// first, which leaves one cut, and are added to the accumulators by float32
+// additions; these are added over the warps in float32 and over the groups as
+// float pairs (k_reduce_groups).  Sums of one sign over 1, 16, 64 and 256
+// images of 256^2 are off by 5e-8 of their value throughout; with the tiles'
+// steps in one accumulator they were by 4e-7, 2.7e-6 and 1e-5 (64 images), by
+// 2e-7 in the FP32 kernel before (serial FP32 sums over 4096 pixels).  Both
+// operands lie in shared memory pixel by pixel, so fragments are read
+// transposed (ldmatrix.trans), a tap being a shift of the pixel rows; the next
+// tile's loads fly while one is multiplied.
+// 16 images of 256^2, all layers: 3.6 ms in FP32, 0.86 ms here.
 __global__ void __launch_bounds__(256) k_conv3_dw(const bf16* __restrict__ in, int Cin, const float* __restrict__ g,
                                                   int Cout, float* __restrict__ part, int B, int H, int Wd,
                                                   int tiles_per_group) {
@@ -531,10 +536,14 @@ __global__ void __launch_bounds__(256) k_conv3_dw(const bf16* __restrict__ in, i
             uint32_t a[4];
             ldmatrix4t(a, aoff + ((t / 3) * PX + t % 3) * CROW);
 #pragma unroll
-            for (int n = 0; n < 2; ++n)
+            for (int n = 0; n < 2; ++n) {
+                float d[4] = {0.f, 0.f, 0.f, 0.f};          // this tile's sums, the smallest parts first
 #pragma unroll
-                for (int u = 0; u < 3; ++u)
-                    mma_bf16_16816(acc[t][n], a[0], a[1], a[2], a[3], w[u][2 * n], w[u][2 * n + 1]);
+                for (int u = 2; u >= 0; --u)
+                    mma_bf16_16816(d, a[0], a[1], a[2], a[3], w[u][2 * n], w[u][2 * n + 1]);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[t][n][v] += d[v];
+            }
         }
         __syncthreads();
     }

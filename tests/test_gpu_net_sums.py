@@ -78,3 +78,29 @@ def test_infinite_gradient(lm):
     gy[77] = np.inf
     g = _grads(lm, (8, 8, 8, 8), 512, gy)
     assert np.all(g["o"] == np.inf) and np.all(g["d0"] == np.inf)
+
+
+# One cut of a tile's sum (below 2^-23 of it, always to one side), and random
+# roundings of 2^-24 in some two dozen additions a warp and group: 2^-23 + 5 2^-24.
+@pytest.mark.parametrize("B,n", [(1, 64), (16, 256)])
+def test_weight_gradient_of_one_sign(lm, B, n):
+    ch = (8, 8, 8, 8)
+    P = U.init_params(np.random.default_rng(0), cin=3, ch=ch)
+    for k, v in P.items():
+        v[:] = 1.0 if k in ("O", "d0") else 0.0
+    for c in range(8):                               # D0's input is the image's channel c % 3
+        P["A0"][1, 1, c % 3, c] = P["B0"][1, 1, c, c] = P["C0"][1, 1, 8 + c, c] = 1.0
+    g = torch.Generator(device="cuda").manual_seed(B)
+    x = torch.rand((B, n, n, 3), device="cuda", generator=g).mul_(0.9).add_(0.1).to(torch.bfloat16).float()
+    gy = torch.rand((B, n, n), device="cuda", generator=g).add_(0.5)
+    net = lm.Net(ch)
+    net.set_params(U.flat_params(P, 3, ch))
+    net.forward(x.reshape(-1), torch.empty(gy.numel(), device="cuda"), B, n, n)
+    net.backward(gy.reshape(-1))
+    got = U.unflat_params(net.grads(), 3, ch)["D0"]
+    net.close()
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 1, 1, 1, 1))
+    for t in range(9):
+        want = (xp[:, t // 3:t // 3 + n, t % 3:t % 3 + n] * gy.double()[..., None]).sum((0, 1, 2)).cpu().numpy()
+        want = want[np.arange(8) % 3][:, None]
+        assert np.all(np.abs(got[t // 3, t % 3] - want) <= 7 * 2.0 ** -24 * want), t
