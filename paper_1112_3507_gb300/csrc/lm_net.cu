@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(256) k_reduce_groups(const float* __restrict__
     if (i < n)
 #pragma unroll 4
         for (int k = threadIdx.y; k < ngroups; k += 8) ff_add(s, part[(size_t)k * n + i]);
-    sm[threadIdx.y][threadIdx.x] = ff_value(s);
+    sm[threadIdx.y][threadIdx.x] = isfinite(s.hi) ? ff_value(s) : (double)s.hi;   // an infinity's error is NaN
     __syncthreads();
     if (threadIdx.y == 0 && i < n) {
         double v = 0.0;

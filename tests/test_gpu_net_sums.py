@@ -75,9 +75,10 @@ def test_bias_gradients_past_float32(lm, names, n, e):
 
 def test_infinite_gradient(lm):
     gy = np.ones(512 * 512, dtype=np.float32)
-    gy[77] = np.inf
+    gy[100 * 512 + 77] = np.inf                      # inside: no zero beside it
     g = _grads(lm, (8, 8, 8, 8), 512, gy)
-    assert np.all(g["o"] == np.inf) and np.all(g["d0"] == np.inf)
+    for k in ("o", "O", "d0", "D0"):
+        assert np.all(g[k] == np.inf), k
 
 
 # One cut of a tile's sum (below 2^-23 of it, always to one side), and random
