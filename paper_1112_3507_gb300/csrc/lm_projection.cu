@@ -20,8 +20,7 @@
 // consecutive); face arrays hold each cell's minus face per axis.  One
 // thread per cell; the float64 pipe bounds these kernels on GB300, so their
 // quotients, five an axis, run on the integer pipe (lm_intfp.cuh): 96^3
-// right-hand side 400 -> 97 us, update 311 -> 128 us, and with the face factor
-// one constant 15 % less (256^2 12.9 -> 10.9 us).
+// right-hand side 400 -> 97 us, update 311 -> 128 us.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -109,6 +108,12 @@ __global__ void __launch_bounds__(lm::NT) k_projection_rhs(ProjGeo G, double dt,
     }
 }
 
+// dt dP ih 2 / s, its products from the left: dt / h alone may leave the range
+// that dt dP stays in.  The doubling is one to the exponent, on the integer pipe.
+__device__ __forceinline__ double face_step(double dt, double dP, double ih, double s) {
+    return lm::idiv(lm::mul_pow2(dt * dP * ih, 2.0, 1), s);
+}
+
 __global__ void __launch_bounds__(lm::NT) k_projection_update(ProjGeo G, double dt, const double* __restrict__ P,
                                                               const double* __restrict__ rho_n,
                                                               const double* __restrict__ m_s,
@@ -125,17 +130,15 @@ __global__ void __launch_bounds__(lm::NT) k_projection_update(ProjGeo G, double 
         double div = 0.0, ugp = 0.0;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double k = 2.0 * dt * G.ih[a];
             const double* ua = uf_s + (size_t)a * N;
             double um = 0.0, mnew = m_s[(size_t)a * N + idx];
             if (ax[a].live) {
                 const double gp = grad_axis(ax[a], idx, P, rho_n, G.ih[a]);
                 mnew -= dt * gp;                                         // Eq. momupdate
                 // step (vii) on the minus and plus faces
-                um = ax[a].wm ? 0.0
-                              : ua[idx] - lm::idiv(k * (Pc - P[ax[a].m]), rn + rho_n[ax[a].m]);
+                um = ax[a].wm ? 0.0 : ua[idx] - face_step(dt, Pc - P[ax[a].m], G.ih[a], rn + rho_n[ax[a].m]);
                 const double up = ax[a].wp ? 0.0
-                                           : ua[ax[a].p] - lm::idiv(k * (P[ax[a].p] - Pc), rho_n[ax[a].p] + rn);
+                                           : ua[ax[a].p] - face_step(dt, P[ax[a].p] - Pc, G.ih[a], rho_n[ax[a].p] + rn);
                 div += (up - um) * G.ih[a];
                 ugp += lm::idiv(mnew, rn) * gp;
             }

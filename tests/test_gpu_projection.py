@@ -123,3 +123,30 @@ def test_fractional_step_projection_on_gpu(lm, shape, bc):
     ufs = [a.reshape(shape) for a in np.split(uf.cpu().numpy(), 3)]
     scale = np.abs(J.divergence(ufs, h, bc)).max()
     assert np.max(np.abs(div - want)) <= 1e-7 * scale
+
+
+# Powers of ten that leave float64's range as dt / h alone, or fall below its
+# normal numbers, while dt (P_c - P_m) / h is an ordinary number; and ordinary
+# ones.  The products are taken from the left, so the face velocities are the
+# bits of that expression.
+@pytest.mark.parametrize("dt,h,dp", [(1e-3, 1.0 / 48, 1.0), (1e299, 1e-10, 1e-295), (1e-300, 1e12, 1e307)])
+@pytest.mark.parametrize("shape,bc", CASES)
+def test_face_update_to_the_bit(lm, shape, bc, dt, h, dp):
+    nz, ny, nx = shape
+    n, hs = (nx, ny, nz), (h, 1.25 * h, 0.75 * h)
+    rng = np.random.default_rng(nx + nz)
+    N = nx * ny * nz
+    P, rho = dp * rng.standard_normal(shape), rng.uniform(0.5, 2.0, shape)
+    uf = rng.standard_normal((3,) + shape)
+    zero = np.zeros(shape)
+    m_new, uf_new, e_new = (torch.empty(k * N, dtype=torch.float64, device="cuda") for k in (3, 3, 1))
+    lm.projection_update(n, hs, bc, dt, _d(P), _d(rho), _v([zero] * 3), _d(uf), _d(zero), m_new, uf_new, e_new)
+    got = uf_new.cpu().numpy().reshape((3,) + shape)
+    for a in range(3):
+        ax = 2 - a
+        if shape[ax] == 1:
+            continue
+        want = uf[a] - dt * (P - np.roll(P, 1, ax)) * (1.0 / hs[a]) * 2.0 / (rho + np.roll(rho, 1, ax))
+        if bc[a] == NEUMANN:
+            want[tuple(0 if k == ax else slice(None) for k in range(3))] = 0.0
+        assert np.array_equal(got[a], want), a
