@@ -194,6 +194,14 @@ __device__ __forceinline__ T bx_point(int idx, const FeOp<T>& op, LD ld, T& xc) 
     return op.vc[idx] * xc + st;
 }
 
+// whether element d (bits: dx, dy, dz of its lowest corner) holds point o (base 3:
+// ox + 1, oy + 1, oz + 1)
+__device__ constexpr bool fe_shares(int o, int d) {
+    const int ox = o % 3 - 1, oy = o / 3 % 3 - 1, oz = o / 9 - 1, dx = d & 1, dy = d >> 1 & 1, dz = d >> 2;
+    return !((ox == 1 && dx) || (ox == -1 && !dx) || (oy == 1 && dy) || (oy == -1 && !dy) || (oz == 1 && dz) ||
+             (oz == -1 && !dz));
+}
+
 // The same in 3D and float64 with the stiffness sums in integers (lm_intfp.cuh),
 // one a class, or one for the three classes of edges where their c is the same
 // (cubic elements).  The float64 form takes 82 issue slots of its pipe a point, at
@@ -211,18 +219,31 @@ __device__ __forceinline__ double bx3_fix(int idx, const FeOp<double>& op, const
     const int pz[3] = {wrap_m(k, g.nz) * sz, k * sz, wrap_p(k, g.nz) * sz};
     uint64_t X[27], E[2][2][2];
     lm::ExpRange rx, re;
+    auto used = [](int o) { return o == 13 || FACES || (o % 3 != 1) + (o / 3 % 3 != 1) + (o / 9 != 1) > 1; };
 #pragma unroll
     for (int o = 0; o < 27; ++o)
-        if (o == 13 || FACES || (o % 3 != 1) + (o / 3 % 3 != 1) + (o / 9 != 1) > 1) {
-            X[o] = (uint64_t)__double_as_longlong(x[pz[o / 9] + ry[o / 3 % 3] + cx[o % 3]]);
-            rx.add((uint32_t)(X[o] >> 32) & 0x7fffffffu);
-        }
+        if (used(o)) X[o] = (uint64_t)__double_as_longlong(x[pz[o / 9] + ry[o / 3 % 3] + cx[o % 3]]);
+    bool wall = false;                                 // some element has no weight
 #pragma unroll
     for (int d = 0; d < 8; ++d) {
         uint64_t& e = E[d >> 2][d >> 1 & 1][d & 1];
         e = (uint64_t)__double_as_longlong(op.ke[pz[1 - (d >> 2)] + ry[1 - (d >> 1 & 1)] + cx[1 - (d & 1)]]);
         re.add((uint32_t)(e >> 32));
+        wall |= !e;
     }
+    if (wall)
+#pragma unroll
+        for (int o = 0; o < 27; ++o)
+            if (o != 13 && used(o)) {
+                uint64_t w = 0;                        // the elements that the two points share
+#pragma unroll
+                for (int d = 0; d < 8; ++d)
+                    if (fe_shares(o, d)) w |= E[d >> 2][d >> 1 & 1][d & 1];
+                X[o] = lm::fix_live(X[o], w, X[13]);
+            }
+#pragma unroll
+    for (int o = 0; o < 27; ++o)
+        if (used(o)) rx.add((uint32_t)(X[o] >> 32) & 0x7fffffffu);
     if (!lm::fix_ok(rx, XB, re, GB)) {
         double xc;
         return bx_point(idx, op, [&](int j) { return x[j]; }, xc);
@@ -241,12 +262,9 @@ __device__ __forceinline__ double bx3_fix(int idx, const FeOp<double>& op, const
             lm::Limbs K{0, 0};
 #pragma unroll
             for (int d = 0; d < 8; ++d) {
-                const int dx = d & 1, dy = d >> 1 & 1, dz = d >> 2;
-                if ((ox == 1 && dx) || (ox == -1 && !dx) || (oy == 1 && dy) || (oy == -1 && !dy) || (oz == 1 && dz) ||
-                    (oz == -1 && !dz))
-                    continue;
-                K.h += L[dz][dy][dx].h;
-                K.l += L[dz][dy][dx].l;
+                if (!fe_shares(o, d)) continue;
+                K.h += L[d >> 2][d >> 1 & 1][d & 1].h;
+                K.l += L[d >> 2][d >> 1 & 1][d & 1].l;
             }
             // (B x)_i holds x_{i+o} - x_i: the sign goes to the class's factor
             s.mac(lm::fix_diff<XB>(c0, X[o], ex), K);

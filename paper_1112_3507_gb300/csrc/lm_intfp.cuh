@@ -189,7 +189,9 @@ LM_HD uint64_t minmod_bits(uint64_t a, uint64_t b) {
 // difference is at least E / 2 in magnitude, and the float64 form rounds it, its
 // product and the partial sums after that by up to 2^-53 of them each -- with XB = 5
 // 8 times the cut for as large a weight.  So x of any spread are taken where the
-// weights lie within a factor of four; all else takes the float64 form.
+// weights lie within a factor of four; all else takes the float64 form.  E has to
+// be the centre's or one that some weight meets: the centre's value stands for a
+// neighbour without weight (past a wall), whose size would cut the others off.
 //
 // Room: |xl|, |xh| < 2^29 with XB <= 5, so differences < 2^30; gl < 2^29 and
 // gh < 2^(24 + GB) <= 2^28.  Six single weights, or FE's sums of two (four terms) and
@@ -211,6 +213,12 @@ LM_HD bool fix_ok(const ExpRange& x, int xb, const ExpRange& g, int gb) {
     const int ex = x.top(), eg = g.top(), sg = g.spread();
     return ex >= 200 && ex < 2047 && eg >= 200 && eg < 2047 && sg <= gb && (x.spread() <= xb || sg <= 1) &&
            (unsigned)(ex + eg - 1023 - 150) < 1880u;
+}
+// x of a neighbour of weight w (the bits of one, or of all of several, or-ed), or
+// the centre's c where that is zero: the term stays zero.  An infinity or NaN stays:
+// it times zero is NaN.
+LM_HD uint64_t fix_live(uint64_t x, uint64_t w, uint64_t c) {
+    return (w << 1) || (x >> 52 & 0x7ff) == 0x7ff ? x : c;
 }
 struct Limbs {
     int32_t h, l;

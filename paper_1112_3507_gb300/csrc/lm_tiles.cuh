@@ -43,12 +43,19 @@ __device__ __forceinline__ double apply64_fix(int idx, const Geo& g, const Op64&
     cell_coords(idx, g, i, j, k);
     const bool y = g.ny > 1;
     const Nbr nx = nbr_x(idx, i, g), nz = nbr_z(idx, k, g), ny = y ? nbr_y(idx, j, g) : nx;
+    // past a wall the cell's own value stands for the wrapped one, whose size has
+    // no place in the row's range (its weight is zero)
+    const int xm = face_minus(i, g.nx, g.bcx) ? nx.im : idx, xp = face_plus(i, g.nx, g.bcx) ? nx.ip : idx;
     const double xc = x[idx];
     const uint64_t uc = dbits(xc);
     uint64_t X[4], W[4];
     auto ld = [](const double* p, int q) { return (uint64_t)__double_as_longlong(p[q]); };
-    X[0] = ld(x, nx.im), X[1] = ld(x, nx.ip), W[0] = ld(op.gx, idx), W[1] = ld(op.gx, nx.ip);
-    if (y) X[2] = ld(x, ny.im), X[3] = ld(x, ny.ip), W[2] = ld(op.gy, idx), W[3] = ld(op.gy, ny.ip);
+    X[0] = ld(x, xm), X[1] = ld(x, xp), W[0] = ld(op.gx, idx), W[1] = ld(op.gx, nx.ip);
+    if (y) {
+        X[2] = ld(x, face_minus(j, g.ny, g.bcy) ? ny.im : idx);
+        X[3] = ld(x, face_plus(j, g.ny, g.bcy) ? ny.ip : idx);
+        W[2] = ld(op.gy, idx), W[3] = ld(op.gy, ny.ip);
+    }
     const double c = op.ct[idx], zm = x[nz.im], zp = x[nz.ip], wm = op.gz[idx], wp = op.gz[nz.ip];
     ExpRange rx, rw;
     rx.add((uint32_t)(uc >> 32) & 0x7fffffffu);
