@@ -78,6 +78,7 @@ struct FeOp {
     FeGeo g;
     T c[8];                  // c(o) by class: bit 0 x, bit 1 y, bit 2 z nonzero
     int faces;               // c of the single-axis classes nonzero
+    int strong;              // classes (1 << class) whose |c| is within four of the largest
     const T* ke;             // element kappa by lowest corner
     const T* vc;             // V c~
     const T* dinv;           // 1 / diag(B)
@@ -244,7 +245,20 @@ __device__ __forceinline__ double bx3_fix(int idx, const FeOp<double>& op, const
 #pragma unroll
     for (int o = 0; o < 27; ++o)
         if (used(o)) rx.add((uint32_t)(X[o] >> 32) & 0x7fffffffu);
-    if (!lm::fix_ok(rx, XB, re, GB)) {
+    lm::ExpRange rs = rx;
+    if (FACES) {                                       // (without faces' weights the c are all the same)
+        uint32_t top[8] = {};
+#pragma unroll
+        for (int o = 0; o < 27; ++o) {
+            uint32_t& t = top[(o % 3 != 1) | (o / 3 % 3 != 1) << 1 | (o / 9 != 1) << 2];
+            t = max(t, (uint32_t)(X[o] >> 32) & 0x7fffffffu);
+        }
+        rs.hi = top[0];
+#pragma unroll
+        for (int cls = 1; cls < 8; ++cls)
+            if (op.strong >> cls & 1) rs.hi = max(rs.hi, top[cls]);
+    }
+    if (!lm::fix_ok(rx, XB, re, GB, rs)) {
         double xc;
         return bx_point(idx, op, [&](int j) { return x[j]; }, xc);
     }
@@ -687,7 +701,7 @@ struct lm_fe {
     FeGeo geo{};
     double c[8] = {0};
     double kd = 0.0;           // K_ref's diagonal entry
-    int faces = 1;
+    int faces = 1, strong = 0;
     int KZ = 1;                // planes a block of the column kernel
     lm_grid* fv = nullptr;     // cell-centred grid on the same points (the preconditioner's hierarchy)
     double *ke = nullptr, *vc = nullptr, *dinv = nullptr;
@@ -723,6 +737,7 @@ FeOp<T> fe_op(const lm_fe* fe) {
     op.g = fe->geo;
     for (int q = 0; q < 8; ++q) op.c[q] = (T)fe->c[q];
     op.faces = fe->faces;
+    op.strong = fe->strong;
     if (sizeof(T) == sizeof(double)) {
         op.ke = (const T*)fe->ke;
         op.vc = (const T*)fe->vc;
@@ -1057,6 +1072,9 @@ int lm_fe_create(int ndim, const int64_t n[3], const double h[3], const int bc[3
     const double tiny = 1e-14 * std::fabs(fe->kd);
     fe->faces = (std::fabs(fe->c[1]) > tiny || std::fabs(fe->c[2]) > tiny || std::fabs(fe->c[4]) > tiny) ? 1 : 0;
     if (!fe->faces) fe->c[1] = fe->c[2] = fe->c[4] = 0.0;
+    double cmax = 0.0;
+    for (int cls = 1; cls < 8; ++cls) cmax = std::max(cmax, std::fabs(fe->c[cls]));
+    for (int cls = 1; cls < 8; ++cls) fe->strong |= (4.0 * std::fabs(fe->c[cls]) >= cmax) << cls;
     fe->KZ = fe_planes(fe->geo);
     const size_t N = fe->N;
     int rc = lm_grid_create(ndim, n, h, bc, &fe->fv);

@@ -192,6 +192,10 @@ LM_HD uint64_t minmod_bits(uint64_t a, uint64_t b) {
 // weights lie within a factor of four; all else takes the float64 form.  E has to
 // be the centre's or one that some weight meets: the centre's value stands for a
 // neighbour without weight (past a wall), whose size would cut the others off.
+// Where classes of neighbours have factors of their own, E has to be, but for one
+// bit, the centre's or one of a strong class, with a factor within four of the
+// largest: if it is the centre's, a cut x is in a difference of about E itself;
+// if not, the difference that holds E has a factor to match every cut one's.
 //
 // Room: |xl|, |xh| < 2^29 with XB <= 5, so differences < 2^30; gl < 2^29 and
 // gh < 2^(24 + GB) <= 2^28.  Six single weights, or FE's sums of two (four terms) and
@@ -208,12 +212,14 @@ struct ExpRange {
     LM_HD int spread() const { return (int)(hi >> 20) - (int)((lo + 1u) >> 20); }
 };
 // both ranges in reach, and the sum's exponent in the normal range however far
-// its terms cancel (zeros are below every scale: 2^200 over the smallest normal)
-LM_HD bool fix_ok(const ExpRange& x, int xb, const ExpRange& g, int gb) {
+// its terms cancel (zeros are below every scale: 2^200 over the smallest normal);
+// strong: the range of the centre and the strong classes
+LM_HD bool fix_ok(const ExpRange& x, int xb, const ExpRange& g, int gb, const ExpRange& strong) {
     const int ex = x.top(), eg = g.top(), sg = g.spread();
-    return ex >= 200 && ex < 2047 && eg >= 200 && eg < 2047 && sg <= gb && (x.spread() <= xb || sg <= 1) &&
-           (unsigned)(ex + eg - 1023 - 150) < 1880u;
+    return ex >= 200 && ex < 2047 && eg >= 200 && eg < 2047 && sg <= gb &&
+           (x.spread() <= xb || (sg <= 1 && strong.top() >= ex - 1)) && (unsigned)(ex + eg - 1023 - 150) < 1880u;
 }
+LM_HD bool fix_ok(const ExpRange& x, int xb, const ExpRange& g, int gb) { return fix_ok(x, xb, g, gb, x); }
 // x of a neighbour of weight w (the bits of one, or of all of several, or-ed), or
 // the centre's c where that is zero: the term stays zero.  An infinity or NaN stays:
 // it times zero is NaN.

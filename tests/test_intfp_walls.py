@@ -1,6 +1,7 @@
 """Integer stencil sums beside walls: a neighbour of no weight, whatever its size,
 leaves the row's accuracy alone (arithmetic on the host; the solvers' refinement
-residuals on the device)."""
+residuals on the device); and rows whose classes of neighbours have factors of
+their own, as finite elements of unequal sides have."""
 import os
 import shutil
 import subprocess
@@ -64,12 +65,72 @@ int main() {
 """
 
 
-def test_rows_beside_walls_on_the_host(tmp_path):
+CLASSES = r"""
+#include <algorithm>
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+#include "lm_intfp.cuh"
+static uint64_t bits(double d) { uint64_t u; memcpy(&u, &d, 8); return u; }
+static double value(uint64_t u) { double d; memcpy(&d, &u, 8); return d; }
+int main() {
+    std::mt19937_64 g(13);
+    double ei = 0, ef = 0, mi = 0, mf = 0;
+    long n = 0;
+    for (long i = 0; i < 1500000; ++i) {         // three classes of four neighbours, factors 2^-12 to 2
+        double x[13], w[12], c[3];
+        auto mant = [&] { return value((g() & ((1ull << 52) - 1)) | 1023ull << 52); };
+        const int spread = 6 + (int)(g() % 50);
+        for (int o = 0; o < 13; ++o) {           // any spread, or one class far above the rest
+            const int e = i % 4 ? (int)(g() % spread) : o < 4 && g() % 4 == 0 ? spread : (int)(g() % 4);
+            x[o] = ldexp(mant(), e) * (g() & 1 ? -1 : 1);
+        }
+        for (int o = 0; o < 12; ++o) w[o] = mant();
+        for (int q = 0; q < 3; ++q) c[q] = ldexp(mant(), -(int)(g() % 12));
+        const double cm = std::max(c[0], std::max(c[1], c[2]));
+        lm::ExpRange rx, rw, rs;
+        auto h = [](double v) { return (uint32_t)(bits(v) >> 32) & 0x7fffffffu; };
+        for (int o = 0; o < 13; ++o) {
+            rx.add(h(x[o]));
+            if (o == 12 || 4.0 * c[o / 4] >= cm) rs.add(h(x[o]));
+        }
+        for (int o = 0; o < 12; ++o) rw.add(h(w[o]));
+        if (rx.spread() <= 5 || !lm::fix_ok(rx, 5, rw, 3, rs)) continue;
+        const lm::Limbs cc = lm::fix<5>(bits(x[12]), rx.top());
+        double yi = 0, yf = 0;
+        long double S = 0, mag = 0;
+        for (int q = 0; q < 3; ++q) {
+            lm::FixSum s;
+            double a = 0;
+            for (int o = 4 * q; o < 4 * q + 4; ++o) {
+                s.mac(lm::fix_diff<5>(cc, bits(x[o]), rx.top()), lm::fix_abs<3>(bits(w[o]), rw.top()));
+                a = fma(w[o], x[12] - x[o], a);
+                const long double t = (long double)c[q] * w[o] * ((long double)x[12] - x[o]);
+                S += t, mag += fabsl(t);
+            }
+            yi = fma(c[q], value(lm::fix_round(s.total(), lm::fix_scale<5, 3>(rx.top(), rw.top()))), yi);
+            yf = fma(c[q], a, yf);
+        }
+        const double a = fabsl(yi - S) / mag, b = fabsl(yf - S) / mag;
+        ei += a, ef += b, ++n;
+        mi = std::max(mi, a), mf = std::max(mf, b);
+    }
+    printf("%ld rows: mean %g against %g, largest %g against %g\n", n, ei / n, ef / n, mi, mf);
+    return !(n > 500000 && ei <= ef && mi <= mf);
+}
+"""
+
+
+# The rows that the integer form takes are as close to the exact sum as the float64
+# form's, on average and at worst.
+@pytest.mark.parametrize("program", [PROGRAM, CLASSES], ids=["walls", "classes"])
+def test_rows_on_the_host(tmp_path, program):
     gxx = shutil.which("g++")
     if not gxx:
         pytest.skip("no g++")
     src, exe = tmp_path / "q.cpp", tmp_path / "q"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     subprocess.run([gxx, "-O2", "-std=c++17", "-I", CSRC, "-o", str(exe), str(src)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout
