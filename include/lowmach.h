@@ -106,7 +106,13 @@ typedef struct {
     double inner_rtol;      /* relative reduction asked of each inner solve      */
     int    inner_max_iter;  /* inner iterations per refinement step               */
     int    check_every;     /* Krylov iterations between host convergence checks
-                               (float64 modes).  Mixed modes check the inner
+                               (float64 modes).  Jacobi-PCG on a grid of up to
+                               2048 cells an SM runs inside one cooperative
+                               kernel, which tests every iteration itself and
+                               returns to the host after at most 1024 of them,
+                               unless check_every == 1 (the same iterates, one
+                               kernel launch per step of the iteration).
+                               Mixed modes check the inner
                                solve on the device (one host check per
                                refinement step) unless check_every == 1: then
                                the host checks after every inner iteration,
@@ -182,6 +188,8 @@ int  lm_load_network(lm_grid* g, const char* weights_path);
 
 /* Solve A P = f (step (vi) of Sec. 2.4) to opts->rtol in the chosen mode.
  * Returns LM_OK, LM_ERR_NO_CONVERGENCE (best iterate kept), LM_ERR_BREAKDOWN,
+ * LM_ERR_TIMEOUT (a block of the cooperative Jacobi-PCG kernel waited some
+ * seconds for another),
  * LM_ERR_STATE (coefficients or rhs missing), LM_ERR_INVALID_ARG (e.g. a
  * multigrid mode on a periodic axis with an odd cell count > 1).  `res` may
  * be NULL.  Synchronises the stream before returning. */
@@ -529,6 +537,13 @@ int  lm_fe_solve(lm_fe* fe, const double* b, double* x, int on_device, const lm_
  * synchronises the stream.  LM_ERR_INVALID_ARG for a bad `which`, `steps`
  * or pointer. */
 int  lm_probe_rate(int which, int steps, double* ops_per_s, void* stream);
+
+/* Limits of the cooperative Jacobi-PCG kernel on this grid: `steps`
+ * iterations (>= 1) between host checks, and `looks` of a waiting block, of
+ * about a microsecond each, before it gives up and the solve returns
+ * LM_ERR_TIMEOUT.  The defaults are 1024 and 2^22; the iterates do not depend
+ * on `steps`. */
+int  lm_jacobi_run_limits(lm_grid* g, int steps, unsigned int looks);
 
 /* Allocation-free float64 apply: y = A x and *dot_out = x^T A x, like
  * lm_apply(LM_PREC_FP64) with dot_out, but with no grid object and no device

@@ -313,17 +313,24 @@ int solve_jacobi_pcg(lm_grid* g, const lm_solve_opts* o, lm_solve_result* res) {
     launch_pcg_init(a, g->G, s, o->use_x0 && g->have_x0);
     CK(cudaGetLastError());
     int k = 0, restarts = 0;
-    // small grids: up to 1024 iterations in one kernel, which stops by itself
-    // (a host check every check_every launches' worth would only slow it)
-    const bool run = g->coop && pcg_run_fits(g->N, g->G, g->nsm);
+    const int chunk = std::max(1, o->check_every);
+    // small grids: up to run_steps iterations in one kernel, which stops by itself
+    // (a host check every check_every launches' worth would only slow it);
+    // check_every = 1 keeps to a launch a step of the iteration
+    bool run = chunk > 1 && g->coop && pcg_run_fits(g->N, g->G, g->nsm);
     if (run && !g->bar && (rc = dalloc(&g->bar, 2))) return rc;
     bool from_part = true;
-    const int chunk = std::max(1, o->check_every);
     if ((rc = sync_state(g, g->st, s))) return rc;
     while (!g->st_host->done) {
         if (run) {
-            const int k1 = (int)std::min<long long>(o->max_iter, (long long)k + 1024);
-            if ((rc = launch_pcg_run(a, g->G, g->nsm, s, k, k1, from_part, g->bar))) return rc;
+            const int k1 = (int)std::min<long long>(o->max_iter, (long long)k + g->run_steps);
+            if (launch_pcg_run(a, g->G, g->nsm, s, k, k1, from_part, g->bar, g->run_looks) != LM_OK) {
+                // refused: the iteration's own launches, which find r.z in the
+                // partials only where a restart puts it there
+                run = false;
+                if (!from_part) launch_pcg_restart(a, g->G, s, k);
+                continue;
+            }
             from_part = false;
         } else {
             for (int c = 0; c < chunk && k < o->max_iter; ++c, ++k) launch_pcg_iter(a, g->G, s, k);
@@ -1054,6 +1061,13 @@ void lm_grid_destroy(lm_grid* g) {
     for (cudaEvent_t e : g->ev_chunk)
         if (e) cudaEventDestroy(e);
     delete g;
+}
+
+int lm_jacobi_run_limits(lm_grid* g, int steps, unsigned int looks) {
+    if (!g || steps < 1) return LM_ERR_INVALID_ARG;
+    g->run_steps = steps;
+    g->run_looks = looks;
+    return LM_OK;
 }
 
 int64_t lm_grid_size(const lm_grid* g) { return g ? (int64_t)g->N : 0; }

@@ -217,17 +217,17 @@ __global__ void __launch_bounds__(NT) k_pcg_p(PcgArgs a, int k) {
 // 81 x 49 x 70: 86.4 -> 35.9 us.  What is left on the small grids is latency:
 // three round trips to L2, three barriers and a chain of some forty dependent
 // float64 steps (operator, sums, quotients).
-constexpr unsigned BAR_LIMIT = 1u << 22;            // looks of about 1 us
 
-// bar[0]: arrivals since the launch; bar[1]: a block gave up.
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& target) {
+// bar[0]: arrivals since the launch; bar[1]: a block gave up, after `looks` looks
+// of about 1 us.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& target, unsigned looks) {
     __shared__ int s_ok;
     __syncthreads();
     target += gridDim.x;
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         int ok = 0;
-        for (unsigned n = 0; n < BAR_LIMIT; ++n) {
+        for (unsigned n = 0; n < looks; ++n) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if (v >= target) {
@@ -310,7 +310,7 @@ __device__ __forceinline__ void pcg_partial(double (&v)[Q], int u, double* part,
 
 template <bool WARPS, int K>
 __global__ void __launch_bounds__(NT, 1) k_pcg_run(PcgArgs a, int G, int k0, int k1, int from_part,
-                                                   unsigned* __restrict__ bar) {
+                                                   unsigned* __restrict__ bar, unsigned looks) {
     constexpr bool KEEP = K <= 4;                   // coefficients in registers
     __shared__ double sm[64];
     // scalars of an iteration: formed by one thread each, since every warp that
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_run(PcgArgs a, int G, int k0, int
             const int sl[1] = {0};
             pcg_partial<WARPS, 1>(acc, u, a.part, sl, sm);
         }
-        if (!(ok = grid_barrier(bar, target))) break;
+        if (!(ok = grid_barrier(bar, target, looks))) break;
         // alpha, x, r, r.r, r.z
         {
             const int sl[1] = {0};
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_run(PcgArgs a, int G, int k0, int
             const int sl[2] = {1, 2 + ((k + 1) & 1)};
             pcg_partial<WARPS, 2>(acc, u, a.part, sl, sm);
         }
-        if (!(ok = grid_barrier(bar, target))) break;
+        if (!(ok = grid_barrier(bar, target, looks))) break;
         // beta, p; the convergence test is formed meanwhile and looked at after
         // the barrier (a p updated past the end is not used)
         {
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_run(PcgArgs a, int G, int k0, int
             }
         }
         rz = rz_new;
-        if (!(ok = grid_barrier(bar, target)) || s_stop) break;
+        if (!(ok = grid_barrier(bar, target, looks)) || s_stop) break;
     }
     if (!ok && tid == 0) {
         a.st->status = LM_ERR_TIMEOUT;
@@ -734,8 +734,9 @@ void launch_pcg_iter(const PcgArgs& a, int G, cudaStream_t s, int k) {
 // block per SM (311,296 cells on 152 SMs), which is also where a launch's
 // blocks stop having one cell a thread.  Larger grids are bound by the float64
 // pipe, not by the launches.
-bool pcg_run_fits(int N, int G, int nsm) { return (long long)G * NT >= N && G <= 8 * nsm ; }
-int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int k1, int from_part, unsigned* bar) {
+bool pcg_run_fits(int N, int G, int nsm) { return (long long)G * NT >= N && G <= 8 * nsm; }
+int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int k1, int from_part, unsigned* bar,
+                   unsigned looks) {
     if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return LM_ERR_CUDA;
     const void* f;
     int blocks = nsm;
@@ -746,9 +747,13 @@ int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int
     else if (G <= 4 * nsm) f = (const void*)k_pcg_run<false, 4>;
     else f = (const void*)k_pcg_run<false, 8>;
     PcgArgs args = a;
-    void* av[] = {&args, &G, &k0, &k1, &from_part, &bar};
+    void* av[] = {&args, &G, &k0, &k1, &from_part, &bar, &looks};
+    if (cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(NT), av, 0, s) != cudaSuccess) {
+        cudaGetLastError();
+        return LM_ERR_CUDA;
+    }
     count_launches(1);
-    return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(NT), av, 0, s) == cudaSuccess ? LM_OK : LM_ERR_CUDA;
+    return LM_OK;
 }
 void launch_true_residual(const PcgArgs& a, int G, cudaStream_t s) {
     count_launches(1);

@@ -53,6 +53,8 @@ struct lm_grid {
     double* scal = nullptr;         // reduction results (float32 kernels)
     unsigned int* ctr = nullptr;    // last-block arrival counter
     unsigned int* bar = nullptr;    // grid barrier of the cooperative Jacobi-PCG kernel (on first use)
+    int run_steps = 1024;           // iterations of that kernel between host checks, at most
+    unsigned run_looks = 1u << 22;  // looks at its barrier before a block gives up (about 1 us each)
     int nsm = 1;                    // SMs of the device
     bool coop = false;              // cooperative launches are available
     double* stage = nullptr;        // 3N host-input staging (allocated on first use)

@@ -102,9 +102,12 @@ void launch_pcg_p(const PcgArgs& a, int G, cudaStream_t s, int k);
 void launch_pcg_iter(const PcgArgs& a, int G, cudaStream_t s, int k);
 // iterations k0 .. k1 - 1 (or until done) in one cooperative kernel, for grids
 // it fits on a device of nsm SMs; from_part: r.z is in the partials (first
-// launch after an init or restart), else in st->scale; bar: two words
+// launch after an init or restart), else in st->scale; bar: two words; looks: of
+// a waiting block at a grid barrier before it gives up.  LM_ERR_CUDA: refused,
+// nothing has run.
 bool pcg_run_fits(int N, int G, int nsm);
-int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int k1, int from_part, unsigned* bar);
+int launch_pcg_run(const PcgArgs& a, int G, int nsm, cudaStream_t s, int k0, int k1, int from_part, unsigned* bar,
+                   unsigned looks);
 void launch_true_residual(const PcgArgs& a, int G, cudaStream_t s);
 void launch_ir_residual(const Geo& g, int G, cudaStream_t s, const Op64& op, const double* f, double* x,
                         float* r32, double* part, int zero_x, SolveState* st, int set_fnorm, double* hist_entry,

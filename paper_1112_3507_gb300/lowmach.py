@@ -68,6 +68,7 @@ _SIGNATURES = {
     "lm_grid_create": (ctypes.c_int, [ctypes.c_int, _I64_3, _D3, _I3, ctypes.POINTER(_P)]),
     "lm_grid_destroy": (None, [_P]),
     "lm_grid_size": (ctypes.c_int64, [_P]),
+    "lm_jacobi_run_limits": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_uint]),
     "lm_set_coefficients": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_double, ctypes.c_int, _P]),
     "lm_set_coefficients_raw": (ctypes.c_int, [_P, _P, _P, ctypes.c_int, _P]),
     "lm_set_rhs": (ctypes.c_int, [_P, _P, ctypes.c_int, _P]),
@@ -299,6 +300,10 @@ class Grid:
         buf = (ctypes.c_double * max(n.value, 1))()
         _check(lib().lm_get_residual_history(self._g, buf, n.value, ctypes.byref(n)), "lm_get_residual_history")
         return np.array(buf[: n.value])
+
+    def jacobi_run_limits(self, steps=1024, looks=1 << 22):
+        """lm_jacobi_run_limits: the cooperative Jacobi-PCG kernel's iterations a launch and looks at a barrier."""
+        _check(lib().lm_jacobi_run_limits(self._g, int(steps), int(looks)), "lm_jacobi_run_limits")
 
     # ---- row-level entry points (device tensors)
     def coefficients(self, stream=None):
