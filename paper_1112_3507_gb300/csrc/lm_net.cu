@@ -168,14 +168,17 @@ __global__ void __launch_bounds__(256) k_conv3_mma(const void* __restrict__ in_,
     const int b = blockIdx.z / nch, co0 = (blockIdx.z % nch) * NCB;
     const int x0 = blockIdx.x * TXP, y0 = blockIdx.y * TYP;
     const int nk = (Cin + 15) / 16;
-    // this thread's half rows: source offset of the pixel (-1: outside the image), half, position
-    int src[QX], dst[QX];
+    // this thread's half rows: the pixel (NONE: outside the image), position
+    constexpr unsigned NONE = ~0u;
+    unsigned src[QX];
+    int dst[QX];
+    const int half = tid & 1;
 #pragma unroll
     for (int q = 0; q < QX; ++q) {
         const int e = tid + 256 * q, pix = e >> 1, py = pix / PX, px = pix - py * PX;
         const int gy = y0 + py - 1, gx = x0 + px - 1;
-        dst[q] = e < 2 * NPIX ? pix * CROW + (e & 1) * 16 : -1;
-        src[q] = dst[q] >= 0 && gy >= 0 && gy < H && gx >= 0 && gx < Wd ? (gy * Wd + gx) * 2 + (e & 1) : -1;
+        dst[q] = e < 2 * NPIX ? pix * CROW + half * 16 : -1;
+        src[q] = dst[q] >= 0 && gy >= 0 && gy < H && gx >= 0 && gx < Wd ? (unsigned)gy * Wd + gx : NONE;
     }
     const size_t img = (size_t)b * H * Wd * Cin;
     constexpr int NV = SPLIT ? 2 : 1;
@@ -185,9 +188,9 @@ __global__ void __launch_bounds__(256) k_conv3_mma(const void* __restrict__ in_,
         for (int q = 0; q < QX; ++q) {
 #pragma unroll
             for (int u = 0; u < NV; ++u) v[q][u] = make_uint4(0, 0, 0, 0);
-            if (src[q] < 0) continue;
-            const int ci = 16 * c + 8 * (src[q] & 1);
-            const size_t at = img + (size_t)(src[q] >> 1) * Cin + ci;
+            if (src[q] == NONE) continue;
+            const int ci = 16 * c + 8 * half;
+            const size_t at = img + (size_t)src[q] * Cin + ci;
             if (Cin % 8 == 0) {
                 if (ci < Cin)
 #pragma unroll
