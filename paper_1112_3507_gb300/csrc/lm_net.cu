@@ -1012,8 +1012,7 @@ struct lm_net {
     bool grads_ready = false;
     bf16 *x = nullptr, *in_[4] = {}, *a1[4] = {}, *e[4] = {}, *cat[3] = {}, *da1[3] = {}, *d[3] = {};
     float* y = nullptr;
-    float *gd0 = nullptr, *gbuf1 = nullptr, *gbuf2 = nullptr, *genc[4] = {}, *gdl[4] = {};
-    bf16* gbf = nullptr;
+    float *gd0 = nullptr, *gbuf1 = nullptr, *gbuf2 = nullptr, *genc[4] = {}, *gdl[3] = {};
     float* part = nullptr;
     size_t part_n = 0;
     double* sums = nullptr;         // per-channel block sums of the backward pass
@@ -1061,7 +1060,9 @@ int ensure_grads(lm_net* N) {
     for (int l = 0; l < 4; ++l) {
         const size_t Pl = P0 >> (2 * l);
         const int cl = N->ch[l];
-        if ((rc = nalloc(N, &N->genc[l], Pl * cl, true)) || (rc = nalloc(N, &N->gdl[l], Pl * cl, true))) return rc;
+        if ((rc = nalloc(N, &N->genc[l], Pl * cl, true))) return rc;
+        // what comes down the decoder: D_0's is gd0, e_3's goes to genc[3]
+        if ((l == 1 || l == 2) && (rc = nalloc(N, &N->gdl[l], Pl * cl, true))) return rc;
     }
     size_t gmax = 0;
     for (int l = 0; l < 4; ++l) {
@@ -1070,11 +1071,11 @@ int ensure_grads(lm_net* N) {
         gmax = std::max(gmax, Pl * (size_t)(l == 0 ? N->cin : N->ch[l - 1]));
     }
     if ((rc = nalloc(N, &N->gd0, P0 * N->ch[0], true)) || (rc = nalloc(N, &N->gbuf1, gmax, true)) ||
-        (rc = nalloc(N, &N->gbuf2, gmax, true)) || (rc = nalloc(N, &N->gbf, gmax, true)))
+        (rc = nalloc(N, &N->gbuf2, gmax, true)))
         return rc;
     N->part_n = 0;
     for (const auto& c : N->convs) N->part_n = std::max(N->part_n, (size_t)9 * c.cin * c.cout);
-    N->part_n *= 256;   // up to 256 pixel groups
+    N->part_n *= 256;   // pixel groups of the largest layer; conv_bwd_w takes more of a smaller one
     if ((rc = nalloc(N, &N->part, N->part_n, true))) return rc;
     int cmax = 1;
     for (int c : N->ch) cmax = std::max(cmax, c);
