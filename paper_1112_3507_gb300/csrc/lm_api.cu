@@ -236,7 +236,7 @@ float* sweep_chain(MgLevel& M, cudaStream_t s, int count, const int* first, cons
 // adjoint order), so the cycle is symmetric for nu1 == nu2.
 void vcycle(lm_grid* g, int l, float* xout, const float* f, int nu1, int nu2, cudaStream_t s) {
     MgLevel& M = g->mg[l];
-    if (l == g->cc_level) {          // the rest of the cycle in one block
+    if (l == g->cc_level) {          // the rest of the cycle in one launch
         size_t smem = 0;
         const CoarseCycle cc = lm::coarse_chain(g, l, g->cc_blocks, true, g->cc_plan, xout, f, nu1, nu2, &smem);
         launch_coarse_cycle(cc, smem, s);
@@ -996,7 +996,7 @@ int lm_grid_create(int ndim, const int64_t n[3], const double h[3], const int bc
         return code;
     };
     if (cudaGetDevice(&g->device) != cudaSuccess) return fail(LM_ERR_CUDA);
-    // the whole-row and one-block coarse-cycle kernels need more than the
+    // the whole-row and one-launch coarse-cycle kernels need more than the
     // default 48 KB of shared memory: allow it before any entry point launches them
     rbgs_row_allow_smem();
     g->cc_blocks = coarse_cycle_allow();

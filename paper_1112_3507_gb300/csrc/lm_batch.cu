@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(256) kb_resid_restrict(const BTask* __restrict
     resid_restrict_tile(V.L, V.C, V.hx, V.hy, V.hz, V.xa, V.f, V.fc, t.bx, t.by, t.bz);
 }
 
-// one block per grid: the grid's coarse V-cycle (its levels from the one-block
-// cycle's first level down), in place of the per-level launches there
+// one block per grid: the grid's coarse V-cycle (lm_coarse.cuh, from the first
+// level that one block can run down), in place of the per-level launches there
 __global__ void __launch_bounds__(CC_THREADS, 1) kb_coarse_cycle(const CoarseCycle* __restrict__ ccs,
                                                         const BGrid* __restrict__ Gs) {
     if (inner_off(Gs[blockIdx.x])) return;
@@ -587,7 +587,7 @@ struct Plan {
     CoarseInv* dinv_items = nullptr;     // the grids' coarsest levels, and the rows of their inverses
     int* dinv_tasks = nullptr;
     int n_inv_tasks = 0;
-    CoarseCycle* dcc = nullptr;          // per-grid one-block coarse cycles (null: per-level launches)
+    CoarseCycle* dcc = nullptr;          // per-grid coarse cycles of one block each (null: per-level launches)
     size_t cc_smem = 0;                  // their dynamic shared memory (the largest chain's)
     float4* dplan = nullptr;             // their plans, formed at every solve
     int max_depth = 0;
@@ -741,7 +741,7 @@ int build_plan(lm_grid* const* grids, int count, const lm_solve_opts* o, cudaStr
             for (int bx = 0; bx < gx; ++bx) tasks.push_back(BTask{i, lev0[i], bx, by, 0, bx + gx * by, gx * gy});
     }
     tap.n = (int)tasks.size() - tap.off;
-    // one-block coarse cycles when every grid's hierarchy has one: the
+    // coarse cycles of one block when every grid's hierarchy has one: the
     // per-level task lists then stop at each grid's coarse-cycle level
     bool fused = true, inverse = true;
     std::vector<int> lstop(count);

@@ -33,6 +33,13 @@
 // a block restricts and prolongs from its own memory: restricted right-hand
 // sides and corrections are stored into their owner's.
 //
+// Registers: the 128 that 512 threads leave each hold four pairs of a 2D level,
+// but not of a 3D one, nor what a cluster's kernel carries beside its own two.
+// By the compiler's count k_coarse_cycle<1, true> spills 148 bytes a thread
+// (176 loaded back), <16, false> 390 (704), <16, true> 666 (1456), partly
+// inside the half-sweeps; <1, false> and kb_coarse_cycle nothing.  What they
+// would take without was not measured.
+//
 // The arithmetic of a level is that of the kernel that sweeps such a level on
 // its own (CCArith), term by term, so a solve's iterates do not depend on
 // where the chain starts.

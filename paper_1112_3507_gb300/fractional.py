@@ -12,8 +12,10 @@ Host-side sequencing only: every step on grid data is one call of the C ABI
   (ix)       lm_eos_ideal          P^{n+1} and c_s^2 from the ideal-gas law
 
 The state (rho, rho u, e, P, c_s^2) stays resident on the device between
-steps; one step costs one host synchronisation (the solve's convergence
-test).
+steps.  One step waits for the device once in lm_set_coefficients (the
+assembly's flags) and several times in lm_solve: once for the state's upload,
+once for the first residual and once a refinement step (in Jacobi-PCG: a check
+of the iterations and one of the true residual).
 """
 from __future__ import annotations
 
