@@ -207,7 +207,7 @@ __device__ constexpr bool fe_shares(int o, int d) {
 // one a class, or one for the three classes of edges where their c is the same
 // (cubic elements).  The float64 form takes 82 issue slots of its pipe a point, at
 // 18.5 cycles an SM; this takes about 750 integer instructions: the residual of
-// 256^3 points 2771 -> 929 us.
+// 256^3 points 2771 -> 941 us.
 template <bool FACES>
 __device__ __forceinline__ double bx3_fix(int idx, const FeOp<double>& op, const double* x) {
     constexpr int XB = 5, GB = 3;

@@ -20,7 +20,7 @@
 // consecutive); face arrays hold each cell's minus face per axis.  One
 // thread per cell; the float64 pipe bounds these kernels on GB300, so their
 // quotients, five an axis, run on the integer pipe (lm_intfp.cuh): 96^3
-// right-hand side 400 -> 97 us, update 311 -> 128 us.
+// right-hand side 400 -> 96 us, update 311 -> 118 us.
 #include <cuda_runtime.h>
 
 #include <cstdio>

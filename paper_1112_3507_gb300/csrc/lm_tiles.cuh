@@ -36,7 +36,7 @@ __device__ __forceinline__ double apply64_at(int idx, const Geo& g, const Op64& 
 // of its instructions, the integer form of two faces about as long as four of them,
 // so the two run side by side.  It wins where the float64 pipe is the bound, in
 // grids of many cells an SM (256^3 residual: 500 us in float64 alone, 400 with all
-// six faces in integers, 333 so); where latency is it makes no difference.
+// six faces in integers, 345 so); where latency is it makes no difference.
 __device__ __forceinline__ double apply64_fix(int idx, const Geo& g, const Op64& op, const double* __restrict__ x) {
     constexpr int XB = 5, GB = 4;
     int i, j, k;
