@@ -2,6 +2,7 @@
 (check_every = 1): the same bits whatever the iterations a launch, over restarts
 and past the host's check; and a wait that runs out."""
 import os
+import threading
 
 import numpy as np
 import pytest
@@ -81,3 +82,23 @@ def test_a_wait_that_runs_out(lm):
         assert g.solve(mode="jacobi", rtol=1e-10, allow=(-5,))["status"] == -5
         g.jacobi_run_limits()
         _same(_solve(g, rtol=1e-10), want)
+
+
+def test_solves_of_several_threads(lm):
+    """Grids of their own on streams of their own: cooperative kernels beside each other."""
+    sizes, bad = [(129, 1, 97), (257, 1, 151), (51, 23, 67), (64, 1, 64)], []
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()), _grid(lm, sizes[k], (PER, PER, WALL), 400.0, seed=k) as g:
+            want = _solve(g, rtol=1e-10, check_every=1)
+            for _ in range(20):
+                got = _solve(g, rtol=1e-10)
+                if got[:3] != want[:3] or not np.array_equal(got[3], want[3]):
+                    bad.append(k)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
