@@ -887,10 +887,6 @@ int lm::chain_level(const lm_grid* g, int nr_max) {
             // as does a 2D level of 128-cell segments under a 3D one
             if (v.arith != CC_INVERSE && march_arith(q)) fits = false;
             if (cc.lev[0].L.g.ny > 1 && v.arith == CC_AXIS) fits = false;
-            // rbgs_tile leaves the first-colour halo cell beside an x wall, or
-            // of a single-cell row, at its old value where a tile ends in y:
-            // another smoother, which such levels keep
-            if (v.arith == CC_FACE && q.ny > 1 && ((q.bcx == LM_BC_NEUMANN && q.ny > 8) || q.nx == 1)) fits = false;
         }
         if (fits) return l;
     }

@@ -655,9 +655,11 @@ __device__ __forceinline__ void rbgs_tile(const Lev32& L, const float* __restric
                 bool oki, okj = true;
                 const int gi = wrap(i0 - 1 + ex1, g.nx, g.bcx, oki);
                 const int gj = HAS_Y ? wrap(j0 - 1 + hyp, g.ny, g.bcy, okj) : 0;
+                // of the unwrapped x, also past a wall: the pair's first cell says
+                // which of the two a plane colours first
+                parc[c] = (i0 - 1 + ex1 + gj) & 1;
                 if (oki && okj) {
                     offc[c] = gi + g.nx * gj;
-                    parc[c] = (gi + gj) & 1;
                     flc[c] = flags(gi, gj);
                 }
             }
