@@ -266,7 +266,8 @@ int  lm_net_get_grads(lm_net* net, float* host, int n);          /* of the last 
 int  lm_net_forward(lm_net* net, const float* x, float* y, int B, int H, int W, void* stream);
 /* parameter gradients of sum(gy * y) for the last forward (overwritten) */
 int  lm_net_backward(lm_net* net, const float* gy, void* stream);
-/* loss = mean((y - t)^2) over n values, gy = its gradient (device); *loss on host if non-NULL */
+/* gy = the gradient of mean((y - t)^2) over n values (device); with loss non-NULL *loss
+ * is that mean, on the host: waits for the stream, and such calls of one net take turns */
 int  lm_net_mse(lm_net* net, const float* y, const float* t, float* gy, long long n, double* loss, void* stream);
 /* one Adam step (Kingma & Ba) with bias correction on the last gradients */
 int  lm_net_adam(lm_net* net, float lr, float beta1, float beta2, float eps, void* stream);
